@@ -16,6 +16,7 @@
 #include "../../include/lbm_em.h"
 #include "common.cuh"
 #include "launchers.h"
+#include "resident.h"
 #include "runtime.h"
 #include "step2.cuh"
 #include "step2_tma.h"
@@ -235,6 +236,14 @@ struct lbm_em {
     bool s4 = false;
     CUtensorMap s4_smap[2], s4_fmap[2], s4_imap;
     StreamPlan s4_plan{}, s4_plan_acc{};  // plain and (FP32) accumulating four-step launches
+    // many steps per launch with the state on chip (small lattices, no step flag): plan, mailboxes
+    // and control words
+    ResidentPlan res{};
+    void *d_mail = nullptr;
+    unsigned *d_ctl = nullptr;
+    bool res_shares = false;         // resident only while no other such handle has steps in flight (others_busy)
+    bool busy = false;               // res_shares: busy_ev marks the end of the steps enqueued last
+    cudaEvent_t busy_ev = nullptr;
     int tma3_ctas = 0;
     int tma_ctas = 0;
     // contour and accumulators
@@ -244,6 +253,7 @@ struct lbm_em {
     int *d_slot = nullptr;
     double *d_acc = nullptr;
     float *d_stage = nullptr;  // four-step accumulation: 12 staged fields per stencil slot
+    void *d_rstage = nullptr;  // resident accumulation: 3 staged fields per stencil slot and step
     ContourPt *d_pts = nullptr;
     double2 *d_inc = nullptr;   // incident E_z phasor at every stencil site (far field)
     double *d_out = nullptr;
@@ -425,12 +435,88 @@ static lbm_em_status build_graph(lbm_em *h, bool acc, cudaGraphExec_t *out) {
     return cuda_status(e, "cudaGraphInstantiate");
 }
 
+// A resident launch takes the whole GPU, a plain one leaves room: several handles that step at the same
+// time on streams of their own fill it together (7 handles, GLUPS with plain / resident launches:
+// FP32 128^2 38 / 22, 256^2 97 / 65, 320^2 99 / 96, 400^2 94 / 132, 512^2 107 / 142; FP64 128^2
+// 15 / 12, 256^2 18.2 / 16.5, 512^2 18.5 / 17.8; double-float 256^2 42 / 18).  So FP32 lattices of at
+// least kResidentAlways sites always take resident launches, the others only on the library's own
+// stream and while no other handle of that kind has steps in flight; a caller's stream keeps its
+// plain launches.  The bits are the same either way.
+static const long long kResidentAlways = 330 * 330;
+static std::mutex g_busy_mu;
+static std::vector<lbm_em *> g_sharing;  // the live handles with res_shares
+
+static bool others_busy(const lbm_em *h) {
+    std::lock_guard<std::mutex> lock(g_busy_mu);
+    // the query is legal whatever other threads capture
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool busy = false;
+    for (lbm_em *o : g_sharing)
+        if (o != h && o->dev == h->dev && o->busy) {
+            o->busy = cudaEventQuery(o->busy_ev) == cudaErrorNotReady;
+            busy = busy || o->busy;
+        }
+    cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return busy;
+}
+
+static void mark_busy(lbm_em *h) {
+    std::lock_guard<std::mutex> lock(g_busy_mu);
+    h->busy = cudaEventRecord(h->busy_ev, h->stream) == cudaSuccess;
+    if (!h->busy) cudaGetLastError();
+}
+
+// n steps (at most kResidentSteps, accumulating kResidentAccSteps) in one resident launch.
+template <typename T>
+static cudaError_t enqueue_resident(lbm_em *h, int n, bool acc) {
+    const int p = h->cur;
+    return launch_resident<T>(make_args<T>(h), (const T *)h->buf[p], (T *)h->buf[1 - p], h->d_time + p,
+                              h->d_time + (1 - p), h->res, h->d_mail, h->d_ctl, n, acc, (T *)h->d_rstage,
+                              acc ? h->ch.n_slots : 0, h->stream);
+}
+
+// Runs of at least this many steps take resident launches (a call of 2 / 3 / 4 steps takes, in us,
+// 13.6 / 19.8 / 25.8 with plain launches and 14 / 16 / 18 with a resident one in FP64 on 64^2;
+// 7.7 / 14 / 13 and 8 / 9 / 10 in FP32 on 256^2).
+static const int kResidentMin = 3;
+
+// Whether the handle's stream is being captured (then the steps are captured as plain launches).
+static bool stream_capturing(const lbm_em *h) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cs != cudaStreamCaptureStatusNone;
+}
+
 // Every FP32 mode gives the same bits (the four-step FP16-deviation launch rounds its stored
 // state once per launch, see step_stream.cu); two-step launches and their graphs start at
 // even t (an odd start takes one single step first), three- and four-step launches anywhere,
 // and a remainder shorter than a launch's steps takes single steps.
 static lbm_em_status run_steps(lbm_em *h, int64_t n, bool acc) {
     const int m = launch_steps(h, acc), gs = graph_steps(h, acc);
+    const bool capable = h->res.ctas > 0 && n >= kResidentMin && !stream_capturing(h);
+    if (capable && !(h->res_shares && others_busy(h))) {
+        const int64_t most = acc ? kResidentAccSteps : kResidentSteps;
+        while (n > 0) {
+            const int c = (int)(n / ((n + most - 1) / most));  // launches of about the same length
+            const cudaError_t e = h->prec == LBM_EM_F64     ? enqueue_resident<double>(h, c, acc)
+                                  : h->prec == LBM_EM_F32X2 ? enqueue_resident<df>(h, c, acc)
+                                                            : enqueue_resident<float>(h, c, acc);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {  // a stream with fewer SMs than the device
+                cudaGetLastError();
+                h->res.ctas = 0;
+                break;
+            }
+            if (lbm_em_status st = cuda_status(e, "resident step launch")) return st;
+            h->cur ^= 1;
+            h->t += c;
+            n -= c;
+        }
+    }
     while (n > 0) {
         const bool even = (h->t & 1) == 0;
         if (h->cur == 0 && n >= gs && (even || m != 2)) {
@@ -457,6 +543,7 @@ static lbm_em_status run_steps(lbm_em *h, int64_t n, bool acc) {
             n -= 1;
         }
     }
+    if (capable && h->res_shares) mark_busy(h);
     return LBM_EM_OK;
 }
 
@@ -468,6 +555,7 @@ static void free_contour(lbm_em *h) {
     dev_free(h, h->d_slot);
     dev_free(h, h->d_acc);
     dev_free(h, h->d_stage);
+    dev_free(h, h->d_rstage);
     dev_free(h, h->d_pts);
     dev_free(h, h->d_inc);
     h->has_contour = false;
@@ -475,6 +563,10 @@ static void free_contour(lbm_em *h) {
 
 static void free_handle(lbm_em *h) {
     if (!h) return;
+    if (h->res_shares) {
+        std::lock_guard<std::mutex> lock(g_busy_mu);
+        g_sharing.erase(std::remove(g_sharing.begin(), g_sharing.end(), h), g_sharing.end());
+    }
     cudaSetDevice(h->dev);
     if (h->stream) {
         free_contour(h);
@@ -487,12 +579,15 @@ static void free_handle(lbm_em *h) {
         dev_free(h, h->d_cs);
         dev_free(h, h->d_out);
         dev_free(h, h->d_fields);
+        dev_free(h, h->d_mail);
+        dev_free(h, h->d_ctl);
         cudaStreamSynchronize(h->stream);  // the pinned blocks are reused by other handles
     }
     if (h->g_plain) cudaGraphExecDestroy(h->g_plain);
     if (h->cap) cudaStreamDestroy(h->cap);
     if (h->stage_ev) cudaEventDestroy(h->stage_ev);
     if (h->up_ev) cudaEventDestroy(h->up_ev);
+    if (h->busy_ev) cudaEventDestroy(h->busy_ev);
     pinned_put(h->h_stage, h->stage_cap);
     pinned_put(h->h_up, h->up_cap);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -638,6 +733,25 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
                 "encoding the tensor maps of a state buffer");
         TRY(encode_id_map(&h->idmap, h->d_mat, h->nx, h->ny, h->pitch, kTmaTileW, kTmaTileH),
             "encoding the tensor map of the ids");
+    }
+    const bool always = h->prec == LBM_EM_F32 && (long long)h->nx * h->ny >= kResidentAlways;
+    if (!step_flags && !h->s4 && h->prec != LBM_EM_F16DEV && (always || h->own_stream)) {
+        TRY(h->prec == LBM_EM_F64     ? resident_plan<double>(h->nx, h->ny, &h->res)
+            : h->prec == LBM_EM_F32X2 ? resident_plan<df>(h->nx, h->ny, &h->res)
+                                      : resident_plan<float>(h->nx, h->ny, &h->res),
+            "planning the resident kernel");
+        if (h->res.ctas > 0) {
+            TRY(dev_alloc(h, &h->d_mail, h->res.mail_bytes), "allocating the mailboxes");
+            TRY(cudaMemsetAsync(h->d_mail, 0, h->res.mail_bytes, h->stream), "cudaMemset");
+            TRY(dev_alloc(h, &h->d_ctl, 2 * sizeof(unsigned)), "allocating the control words");
+            TRY(cudaMemsetAsync(h->d_ctl, 0, 2 * sizeof(unsigned), h->stream), "cudaMemset");
+            if (!always) {
+                TRY(cudaEventCreateWithFlags(&h->busy_ev, cudaEventDisableTiming), "cudaEventCreate");
+                std::lock_guard<std::mutex> lock(g_busy_mu);
+                g_sharing.push_back(h);
+                h->res_shares = true;
+            }
+        }
     }
     TRY(dev_alloc(h, &h->d_mtab, 256 * sizeof(MatT<double>)), "allocating the material table");
     TRY(dev_alloc(h, &h->d_time, 2 * sizeof(long long)), "allocating the time words");
@@ -904,6 +1018,9 @@ lbm_em_status lbm_em_set_contour(lbm_em_t *h, const lbm_em_contour *c) {
     if (!st) st = cuda_status(dev_alloc(h, &h->d_inc, b_inc), "allocating the incident table");
     if (!st && h->s4 && ch.n_slots > 0)
         st = cuda_status(dev_alloc(h, &h->d_stage, (size_t)ch.n_slots * 12 * sizeof(float)),
+                         "allocating the accumulation stage");
+    if (!st && h->res.ctas > 0 && ch.n_slots > 0)
+        st = cuda_status(dev_alloc(h, &h->d_rstage, (size_t)kResidentAccSteps * 3 * ch.n_slots * h->elem),
                          "allocating the accumulation stage");
     char *up = nullptr;
     if (!st) st = cuda_status(upload_staging(h, o_inc + b_inc, (void **)&up), "pinned staging");

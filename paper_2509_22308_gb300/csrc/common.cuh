@@ -101,7 +101,7 @@ __device__ __forceinline__ void source_values(const SourceParams &s, long long t
         const double v = sin(0.5 * 3.14159265358979323846 * (double)t / (double)s.ramp);
         ramp = v * v;
     }
-    *g_open = ramp * (p0 - p1);
+    *g_open = __dmul_rn(ramp, p0 - p1);  // never fused into the sum it enters: the same value in every kernel
     *inc = ramp * p0;
 }
 
