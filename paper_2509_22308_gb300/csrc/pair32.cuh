@@ -73,17 +73,24 @@ __device__ __forceinline__ PairMat pair_mat(const MatT<float> &a, const MatT<flo
                    pack2(-a.c3, -b.c3)};
 }
 
+// moments() (TM) of both sites.
+__device__ __forceinline__ void moments_pair(const Pop<f2> &p, const PairMat &m, f2 &E3, f2 &Hx, f2 &Hy, f2 &d) {
+    const f2 two = both(2.0f);
+    d = add2(add2(add2(fma2(m.cd, p.ez, p.epx), p.emx), p.epy), p.emy);
+    E3 = quot2(d, m.nc3, m.inv3);
+    Hx = add2(fma2(two, p.hxz, add2(p.hxpx, p.hxmx)), sub2(p.epy, p.emy));
+    Hy = add2(fma2(two, p.hyz, add2(p.hypy, p.hymy)), sub2(p.emx, p.epx));
+}
+
 // Moments and collision of both sites.  e3: per site the field (of TE the larger one) whose
 // exponent field decides the runaway test; the exponent field of a maximum over many of them
 // (amax3) is field_runaway() over each.  F3: the field triple of update_site() in FP32 to f3.
 template <int POL, bool F3>
 __device__ __forceinline__ void update_pair(Pop<f2> &p, const PairMat &m, f2 &e3, f2 *f3) {
     const f2 third = both(1.0f / 3.0f), n3 = both(-3.0f), two = both(2.0f);
-    const f2 d = add2(add2(add2(fma2(m.cd, p.ez, p.epx), p.emx), p.epy), p.emy);
-    const f2 E3 = quot2(d, m.nc3, m.inv3);
     if constexpr (POL == POL_TM) {
-        const f2 Hx = add2(fma2(two, p.hxz, add2(p.hxpx, p.hxmx)), sub2(p.epy, p.emy));
-        const f2 Hy = add2(fma2(two, p.hyz, add2(p.hypy, p.hymy)), sub2(p.emx, p.epx));
+        f2 E3, Hx, Hy, d;
+        moments_pair(p, m, E3, Hx, Hy, d);
         e3 = E3;
         if (F3) {
             f3[0] = mul2(d, m.inv);
@@ -103,6 +110,8 @@ __device__ __forceinline__ void update_pair(Pop<f2> &p, const PairMat &m, f2 &e3
         p.hymy = sub2(hy3, p.hymy);
         p.hyz = sub2(hy3, p.hyz);
     } else {
+        const f2 d = add2(add2(add2(fma2(m.cd, p.ez, p.epx), p.emx), p.epy), p.emy);
+        const f2 E3 = quot2(d, m.nc3, m.inv3);
         const f2 dx = add2(add2(add2(fma2(m.cd, p.hxz, p.hxpx), p.hxmx), p.hypy), p.hymy);
         const f2 Ex3 = quot2(dx, m.nc3, m.inv3);
         const f2 Hz = add2(fma2(two, p.hyz, sub2(p.epx, p.emx)), sub2(p.hymy, p.hypy));

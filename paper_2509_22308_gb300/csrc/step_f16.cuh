@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "pair32.cuh"
 
 namespace lbmem {
 
@@ -161,24 +162,29 @@ __device__ __forceinline__ void encode_all(const Pop<float> &p, const Fld &F, fl
     g[P_HYZ] = __float2half_rn(encode_f(p.hyz, q.hy, sc));
 }
 
-// encode_all of two sites at once, site a in the low and site b in the high half of each
-// pair (one paired conversion per population).
-__device__ __forceinline__ void encode_pair(const Pop<float> &a, const Pop<float> &b, const Fld &Fa, const Fld &Fb,
-                                            float sc, __half2 g[NPLANES]) {
-    const EqS qa = eq_scaled(Fa.e, Fa.hx, Fa.hy, sc), qb = eq_scaled(Fb.e, Fb.hx, Fb.hy, sc);
-#define LBMEM_ENC2(P, m, eq) g[P] = __floats2half2_rn(encode_f(a.m, qa.eq, sc), encode_f(b.m, qb.eq, sc))
-    LBMEM_ENC2(P_EZ, ez, z);
-    LBMEM_ENC2(P_EPX, epx, px);
-    LBMEM_ENC2(P_EMX, emx, mx);
-    LBMEM_ENC2(P_EPY, epy, py);
-    LBMEM_ENC2(P_EMY, emy, my);
-    LBMEM_ENC2(P_HXPX, hxpx, hx);
-    LBMEM_ENC2(P_HXMX, hxmx, hx);
-    LBMEM_ENC2(P_HXZ, hxz, hx);
-    LBMEM_ENC2(P_HYPY, hypy, hy);
-    LBMEM_ENC2(P_HYMY, hymy, hy);
-    LBMEM_ENC2(P_HYZ, hyz, hy);
-#undef LBMEM_ENC2
+// encode_all of two sites at once (low halves: site A, high halves: site B) with packed FP32
+// arithmetic and one paired conversion per population.  The equilibria are negated by a product
+// with -1 (exact), so that each population is one packed FMA.
+__device__ __forceinline__ void encode_pair2(const Pop<f2> &p, f2 e3, f2 hx3, f2 hy3, float scale, __half2 g[NPLANES]) {
+    const f2 h = both(0.5f * scale), sc = both(scale), m1 = both(-1.0f);
+    const f2 e = mul2(e3, h), hx = mul2(hx3, h), hy = mul2(hy3, h);
+    const f2 nz = mul2(e, m1), npx = mul2(sub2(e, hy), m1), nmx = mul2(add2(e, hy), m1), npy = mul2(add2(e, hx), m1),
+             nmy = mul2(sub2(e, hx), m1), nhx = mul2(hx, m1), nhy = mul2(hy, m1);
+    auto enc = [&](f2 f, f2 neq) {
+        const f2 v = fma2(f, sc, neq);
+        return __floats2half2_rn(lo2(v), hi2(v));
+    };
+    g[P_EZ] = enc(p.ez, nz);
+    g[P_EPX] = enc(p.epx, npx);
+    g[P_EMX] = enc(p.emx, nmx);
+    g[P_EPY] = enc(p.epy, npy);
+    g[P_EMY] = enc(p.emy, nmy);
+    g[P_HXPX] = enc(p.hxpx, nhx);
+    g[P_HXMX] = enc(p.hxmx, nhx);
+    g[P_HXZ] = enc(p.hxz, nhx);
+    g[P_HYPY] = enc(p.hypy, nhy);
+    g[P_HYMY] = enc(p.hymy, nhy);
+    g[P_HYZ] = enc(p.hyz, nhy);
 }
 
 // What the next step's pull rebuilds from this site (its stored fields and encoded

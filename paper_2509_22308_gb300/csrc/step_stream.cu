@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "pair32.cuh"
 #include "step2_tma.h"
 #include "step_f16.cuh"
 #include "step_stream.h"
@@ -101,63 +102,51 @@ static __device__ __noinline__ SrcLevels source_levels_f(const SourceParams src,
 }
 
 // The nine populations of a row that the next level reads at the row itself or from its x
-// neighbours, for this lane's sites A (even column, [0]) and B (odd column, [1]).  The +y
-// pair is read one row further down, the -y pair one row further up (not kept).
+// neighbours, for this lane's sites A (even column, low half) and B (odd column, high half).  The
+// +y pair is read one row further down, the -y pair one row further up (not kept).
 struct Row9 {
-    float ez[2], epx[2], emx[2], epy[2], hxpx[2], hxmx[2], hxz[2], hypy[2], hyz[2];
+    f2 ez, epx, emx, epy, hxpx, hxmx, hxz, hypy, hyz;
 };
 
-__device__ __forceinline__ void keep_row(Row9 &r, const Pop<float> &a, const Pop<float> &b) {
-    r.ez[0] = a.ez, r.ez[1] = b.ez;
-    r.epx[0] = a.epx, r.epx[1] = b.epx;
-    r.emx[0] = a.emx, r.emx[1] = b.emx;
-    r.epy[0] = a.epy, r.epy[1] = b.epy;
-    r.hxpx[0] = a.hxpx, r.hxpx[1] = b.hxpx;
-    r.hxmx[0] = a.hxmx, r.hxmx[1] = b.hxmx;
-    r.hxz[0] = a.hxz, r.hxz[1] = b.hxz;
-    r.hypy[0] = a.hypy, r.hypy[1] = b.hypy;
-    r.hyz[0] = a.hyz, r.hyz[1] = b.hyz;
+__device__ __forceinline__ void keep_row(Row9 &r, const Pop<f2> &a) {
+    r.ez = a.ez;
+    r.epx = a.epx;
+    r.emx = a.emx;
+    r.epy = a.epy;
+    r.hxpx = a.hxpx;
+    r.hxmx = a.hxmx;
+    r.hxz = a.hxz;
+    r.hypy = a.hypy;
+    r.hyz = a.hyz;
 }
 
 // f_i(q, next time) of sites A and B of this lane from the post-collision values of row q
 // (cur), the +y pair of row q - 1 (ey, hy) and the -y pair of row q + 1 (my, mh).  Along x
 // the upstream site is the adjacent one (across lanes by shuffles), or the site itself at
 // the lattice edge (the zero-gradient open edge).
-__device__ __forceinline__ void pull_row(const Row9 &cur, const float ey[2], const float hy[2], const float my[2],
-                                         const float mh[2], bool xa0, bool xa_last, bool xb_last, Pop<float> &a,
-                                         Pop<float> &b) {
+__device__ __forceinline__ void pull_row(const Row9 &cur, f2 ey, f2 hy, f2 my, f2 mh, bool xa0, bool xa_last, bool xb_last,
+                                         Pop<f2> &a) {
     const unsigned full = 0xffffffffu;
-    const float l_epx = __shfl_up_sync(full, cur.epx[1], 1);    // site B of the lane to the left
-    const float l_hxpx = __shfl_up_sync(full, cur.hxpx[1], 1);
-    const float r_emx = __shfl_down_sync(full, cur.emx[0], 1);  // site A of the lane to the right
-    const float r_hxmx = __shfl_down_sync(full, cur.hxmx[0], 1);
-    a.ez = cur.ez[0];
-    a.hxz = cur.hxz[0];
-    a.hyz = cur.hyz[0];
-    a.epx = xa0 ? cur.epx[0] : l_epx;
-    a.hxpx = xa0 ? cur.hxpx[0] : l_hxpx;
-    a.emx = xa_last ? cur.emx[0] : cur.emx[1];
-    a.hxmx = xa_last ? cur.hxmx[0] : cur.hxmx[1];
-    a.epy = ey[0];
-    a.hypy = hy[0];
-    a.emy = my[0];
-    a.hymy = mh[0];
-    b.ez = cur.ez[1];
-    b.hxz = cur.hxz[1];
-    b.hyz = cur.hyz[1];
-    b.epx = cur.epx[0];
-    b.hxpx = cur.hxpx[0];
-    b.emx = xb_last ? cur.emx[1] : r_emx;
-    b.hxmx = xb_last ? cur.hxmx[1] : r_hxmx;
-    b.epy = ey[1];
-    b.hypy = hy[1];
-    b.emy = my[1];
-    b.hymy = mh[1];
+    const float l_epx = __shfl_up_sync(full, hi2(cur.epx), 1);  // site B of the lane to the left
+    const float l_hxpx = __shfl_up_sync(full, hi2(cur.hxpx), 1);
+    const float r_emx = __shfl_down_sync(full, lo2(cur.emx), 1);  // site A of the lane to the right
+    const float r_hxmx = __shfl_down_sync(full, lo2(cur.hxmx), 1);
+    a.ez = cur.ez;
+    a.hxz = cur.hxz;
+    a.hyz = cur.hyz;
+    a.epx = pack2(xa0 ? lo2(cur.epx) : l_epx, lo2(cur.epx));
+    a.hxpx = pack2(xa0 ? lo2(cur.hxpx) : l_hxpx, lo2(cur.hxpx));
+    a.emx = pack2(xa_last ? lo2(cur.emx) : hi2(cur.emx), xb_last ? hi2(cur.emx) : r_emx);
+    a.hxmx = pack2(xa_last ? lo2(cur.hxmx) : hi2(cur.hxmx), xb_last ? hi2(cur.hxmx) : r_hxmx);
+    a.epy = ey;
+    a.hypy = hy;
+    a.emy = my;
+    a.hymy = mh;
 }
 
 // One plane of a staged FP32 row: the lane's two sites.
-__device__ __forceinline__ float2 lds2(const float *row, int plane, int lane) {
-    return reinterpret_cast<const float2 *>(row + plane * LW)[lane];
+__device__ __forceinline__ f2 lds2(const float *row, int plane, int lane) {
+    return reinterpret_cast<const f2 *>(row + plane * LW)[lane];
 }
 
 template <bool F16>
@@ -187,11 +176,11 @@ struct StreamArgs {
     float *fe_out, *fhx_out, *fhy_out;
 };
 
-__device__ __forceinline__ void store2(float *p, bool two, float a, float b) {
+__device__ __forceinline__ void store2(float *p, bool two, f2 v) {
     if (two)
-        *reinterpret_cast<float2 *>(p) = make_float2(a, b);
+        *reinterpret_cast<f2 *>(p) = v;
     else
-        *p = a;
+        *p = lo2(v);
 }
 
 // Time levels 1..3 of the wavefront: per level the kept row (row i - 1 - k when row i arrives,
@@ -199,7 +188,7 @@ __device__ __forceinline__ void store2(float *p, bool two, float a, float b) {
 // in the ring; index 0 of these arrays is unused.
 struct Wave {
     Row9 cur[BT];
-    float oe[BT][2], oh[BT][2];
+    f2 oe[BT], oh[BT];
     unsigned ids[BT];
 };
 
@@ -215,9 +204,8 @@ __device__ __forceinline__ Fld2 slot_fields(const unsigned char *sl, int lane) {
 __device__ __forceinline__ unsigned slot_dev(const unsigned char *sl, int plane, int lane) {
     return reinterpret_cast<const unsigned *>(reinterpret_cast<const __half *>(sl) + DEVOFF + plane * DEVW)[lane];
 }
-__device__ __forceinline__ void rebuild2(float eq2a, float eq2b, unsigned g2, unsigned short nis, float o[2]) {
-    o[0] = rebuild_h<false>(eq2a, g2, nis);
-    o[1] = rebuild_h<true>(eq2b, g2, nis);
+__device__ __forceinline__ f2 rebuild2(float eq2a, float eq2b, unsigned g2, unsigned short nis) {
+    return pack2(rebuild_h<false>(eq2a, g2, nis), rebuild_h<true>(eq2b, g2, nis));
 }
 
 // One row of level 0 from a slot: FP32 as staged; FP16-deviation rebuilt in place first (see
@@ -303,40 +291,15 @@ struct RingState {
     unsigned ph;
 };
 
-// update_site<POL, true> (common.cuh) with the fields that enter the Fourier sums returned in
-// FP32: f3 holds the values update_site converts to FP64 (the flush kernels convert them).
-template <int POL>
-__device__ __forceinline__ bool update_site_f3(Pop<float> &p, const MatT<float> &m, unsigned rthr, float f3[3]) {
-    bool bad;
-    if constexpr (POL == POL_TM) {
-        float E3, Hx, Hy, D;
-        moments(p, m, &E3, &Hx, &Hy, &D);
-        bad = field_runaway(E3, rthr);
-        f3[0] = D * m.inv_eps;
-        f3[1] = Hx;
-        f3[2] = Hy;
-        collide(p, E3, Hx, Hy);
-    } else {
-        float Ey3, Ex3, Hz, Dy, Dx;
-        moments_te(p, m, &Ey3, &Ex3, &Hz, &Dy, &Dx);
-        bad = field_runaway(Ey3, rthr) || field_runaway(Ex3, rthr);
-        f3[0] = Hz;
-        f3[1] = Dx * m.inv_eps;
-        f3[2] = Dy * m.inv_eps;
-        collide_te(p, Ey3, Ex3, Hz);
-    }
-    return bad;
-}
-
 // ACC: the FP32 fields of one owned stencil site (slot sl >= 0) at level k of the launch, into
 // the staging buffer that a flush kernel adds to the site's Fourier sums (Sec. III: Fourier
 // analysis over one period) after the launch.
-__device__ __forceinline__ void stage_owned(float *stage, int sl, int k, const float f3f[3]) {
+__device__ __forceinline__ void stage_owned(float *stage, int sl, int k, float f0, float f1, float f2) {
     if (sl < 0) return;
     float *s = stage + 12 * (size_t)sl + 3 * k;
-    s[0] = f3f[0];
-    s[1] = f3f[1];
-    s[2] = f3f[2];
+    s[0] = f0;
+    s[1] = f1;
+    s[2] = f2;
 }
 
 // Four steps of one work unit (see the top of this file).  Returns false after a bounded wait
@@ -347,6 +310,13 @@ __device__ __forceinline__ void stage_owned(float *stage, int sl, int k, const f
 // same order and arithmetic as one step per launch.  Adding them here cost a few FP64
 // instructions per stencil site, which on GB300's FP64 pipe made the units along the contour's
 // vertical tangents (a stencil site in every row) the launch's long tail.
+// The lane's two sites are one packed FP32 pair throughout (pair32.cuh): the levels' arithmetic takes half
+// the issue slots.  What bounds the row loop is the latency of its dependent instructions at 2.7
+// warps per scheduler (issue slots 53 % used), not the pipe, so the gain over scalar
+// arithmetic is small: 2048^2 from 200.6 to 209.0 GLUPS, 8192^2 (near the memory's rate) from
+// 239.6 to 242.7, FP16-deviation and batches even.  Keeping a row pair's material constants from
+// level to level (reloaded where a vote finds other ids) spilled and lost: 2048^2 203.0, a batch
+// of 180 instances of 160^2 28 % slower.
 template <bool F16, int POL, bool ACC, bool SPLIT, bool MIX = false>
 __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, RingState &R, bool &bad) {
     // the steady-state copies treat every computed row as owned, which holds for the stored level
@@ -386,8 +356,8 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
     Wave wa;
 #pragma unroll
     for (int k = 0; k < BT; ++k) {
-        keep_row(wa.cur[k], Pop<float>{}, Pop<float>{});
-        wa.oe[k][0] = wa.oe[k][1] = wa.oh[k][0] = wa.oh[k][1] = 0.f;
+        keep_row(wa.cur[k], Pop<f2>{});
+        wa.oe[k] = wa.oh[k] = f2{0ull};
         wa.ids[k] = 0u;
     }
 
@@ -420,14 +390,14 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
                     slots[k] = *reinterpret_cast<const int2 *>(u.slot + (size_t)q * u.pitch + xa);
             }
         }
-        Pop<float> na{}, nb{};  // level k of row i - k, the -y pair for level k + 1
+        Pop<f2> na{};  // level k of row i - k, the -y pair for level k + 1
         bool have = FAST || i < yhi;
         unsigned id_k0 = 0;
 #pragma unroll
         for (int k = 0; k < BT; ++k) {
             const int q = i - 1 - k;
             const bool compute = FAST || (q >= ylo && q < ny);  // uniform over the warp
-            Pop<float> ca{}, cb{};
+            Pop<f2> c{};
             if (compute) {
                 unsigned idq;
                 if (k == 0) {
@@ -438,139 +408,142 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
                     const unsigned char *su = ring + (size_t)(FAST || q > ylo ? s2 : s1) * LY::SLOT;
                     const unsigned char *sd = ring + (size_t)(FAST || q < ny - 1 ? s0 : s1) * LY::SLOT;
                     Row9 c0;
-                    float ey[2], hy[2], my[2], mh[2];
+                    f2 ey, hy, my, mh;
                     if constexpr (F16 && MIX) {
                         // the stored deviations rebuilt where they are read, each with its own row's
                         // fields: row q's seven in-row populations, row q - 1's +y pair, row q + 1's
                         // -y pair (every population of every row is read, and rebuilt, once)
                         const unsigned short nis = u.nis;
                         const Fld2 Q = slot_fields(sq, lane), U = slot_fields(su, lane), D = slot_fields(sd, lane);
-                        rebuild2(Q.e.x, Q.e.y, slot_dev(sq, P_EZ, lane), nis, c0.ez);
-                        rebuild2(eq2_epx(Q.e.x, Q.hx.x, Q.hy.x), eq2_epx(Q.e.y, Q.hx.y, Q.hy.y),
-                                 slot_dev(sq, P_EPX, lane), nis, c0.epx);
-                        rebuild2(eq2_emx(Q.e.x, Q.hx.x, Q.hy.x), eq2_emx(Q.e.y, Q.hx.y, Q.hy.y),
-                                 slot_dev(sq, P_EMX, lane), nis, c0.emx);
-                        rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXPX, lane), nis, c0.hxpx);
-                        rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXMX, lane), nis, c0.hxmx);
-                        rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXZ, lane), nis, c0.hxz);
-                        rebuild2(Q.hy.x, Q.hy.y, slot_dev(sq, P_HYZ, lane), nis, c0.hyz);
-                        rebuild2(eq2_epy(U.e.x, U.hx.x, U.hy.x), eq2_epy(U.e.y, U.hx.y, U.hy.y),
-                                 slot_dev(su, P_EPY, lane), nis, ey);
-                        rebuild2(U.hy.x, U.hy.y, slot_dev(su, P_HYPY, lane), nis, hy);
-                        rebuild2(eq2_emy(D.e.x, D.hx.x, D.hy.x), eq2_emy(D.e.y, D.hx.y, D.hy.y),
-                                 slot_dev(sd, P_EMY, lane), nis, my);
-                        rebuild2(D.hy.x, D.hy.y, slot_dev(sd, P_HYMY, lane), nis, mh);
+                        c0.ez = rebuild2(Q.e.x, Q.e.y, slot_dev(sq, P_EZ, lane), nis);
+                        c0.epx = rebuild2(eq2_epx(Q.e.x, Q.hx.x, Q.hy.x), eq2_epx(Q.e.y, Q.hx.y, Q.hy.y),
+                                          slot_dev(sq, P_EPX, lane), nis);
+                        c0.emx = rebuild2(eq2_emx(Q.e.x, Q.hx.x, Q.hy.x), eq2_emx(Q.e.y, Q.hx.y, Q.hy.y),
+                                          slot_dev(sq, P_EMX, lane), nis);
+                        c0.hxpx = rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXPX, lane), nis);
+                        c0.hxmx = rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXMX, lane), nis);
+                        c0.hxz = rebuild2(Q.hx.x, Q.hx.y, slot_dev(sq, P_HXZ, lane), nis);
+                        c0.hyz = rebuild2(Q.hy.x, Q.hy.y, slot_dev(sq, P_HYZ, lane), nis);
+                        ey = rebuild2(eq2_epy(U.e.x, U.hx.x, U.hy.x), eq2_epy(U.e.y, U.hx.y, U.hy.y),
+                                      slot_dev(su, P_EPY, lane), nis);
+                        hy = rebuild2(U.hy.x, U.hy.y, slot_dev(su, P_HYPY, lane), nis);
+                        my = rebuild2(eq2_emy(D.e.x, D.hx.x, D.hy.x), eq2_emy(D.e.y, D.hx.y, D.hy.y),
+                                      slot_dev(sd, P_EMY, lane), nis);
+                        mh = rebuild2(D.hy.x, D.hy.y, slot_dev(sd, P_HYMY, lane), nis);
                     } else {
                         const float *rq = reinterpret_cast<const float *>(sq);
                         const float *ru = reinterpret_cast<const float *>(su);
                         const float *rd = reinterpret_cast<const float *>(sd);
-                        float2 v;
-                        v = lds2(rq, P_EZ, lane), c0.ez[0] = v.x, c0.ez[1] = v.y;
-                        v = lds2(rq, P_EPX, lane), c0.epx[0] = v.x, c0.epx[1] = v.y;
-                        v = lds2(rq, P_EMX, lane), c0.emx[0] = v.x, c0.emx[1] = v.y;
-                        v = lds2(rq, P_HXPX, lane), c0.hxpx[0] = v.x, c0.hxpx[1] = v.y;
-                        v = lds2(rq, P_HXMX, lane), c0.hxmx[0] = v.x, c0.hxmx[1] = v.y;
-                        v = lds2(rq, P_HXZ, lane), c0.hxz[0] = v.x, c0.hxz[1] = v.y;
-                        v = lds2(rq, P_HYZ, lane), c0.hyz[0] = v.x, c0.hyz[1] = v.y;
-                        v = lds2(ru, P_EPY, lane), ey[0] = v.x, ey[1] = v.y;
-                        v = lds2(ru, P_HYPY, lane), hy[0] = v.x, hy[1] = v.y;
-                        v = lds2(rd, P_EMY, lane), my[0] = v.x, my[1] = v.y;
-                        v = lds2(rd, P_HYMY, lane), mh[0] = v.x, mh[1] = v.y;
+                        c0.ez = lds2(rq, P_EZ, lane);
+                        c0.epx = lds2(rq, P_EPX, lane);
+                        c0.emx = lds2(rq, P_EMX, lane);
+                        c0.hxpx = lds2(rq, P_HXPX, lane);
+                        c0.hxmx = lds2(rq, P_HXMX, lane);
+                        c0.hxz = lds2(rq, P_HXZ, lane);
+                        c0.hyz = lds2(rq, P_HYZ, lane);
+                        ey = lds2(ru, P_EPY, lane);
+                        hy = lds2(ru, P_HYPY, lane);
+                        my = lds2(rd, P_EMY, lane);
+                        mh = lds2(rd, P_HYMY, lane);
                     }
                     if (NOX)
-                        pull_row(c0, ey, hy, my, mh, false, false, false, ca, cb);
+                        pull_row(c0, ey, hy, my, mh, false, false, false, c);
                     else
-                        pull_row(c0, ey, hy, my, mh, xa0, xa_last, xb_last, ca, cb);
+                        pull_row(c0, ey, hy, my, mh, xa0, xa_last, xb_last, c);
                     idq = *reinterpret_cast<const unsigned short *>(sq + LY::IDS + idoff + 2 * lane);
                     id_k0 = idq;
                 } else {
-                    float ey[2], hy[2], my[2], mh[2];
+                    f2 ey, hy, my, mh;
                     if (!FAST && q == 0) {  // top edge: the +y pair of row 0 itself
-                        ey[0] = in.cur[k].epy[0], ey[1] = in.cur[k].epy[1];
-                        hy[0] = in.cur[k].hypy[0], hy[1] = in.cur[k].hypy[1];
+                        ey = in.cur[k].epy, hy = in.cur[k].hypy;
                     } else {
-                        ey[0] = in.oe[k][0], ey[1] = in.oe[k][1], hy[0] = in.oh[k][0], hy[1] = in.oh[k][1];
+                        ey = in.oe[k], hy = in.oh[k];
                     }
                     if (!FAST && q == ny - 1) {  // bottom edge: the -y pair of the last row itself
                         const float4 e = edge[k * 32 + lane];
-                        my[0] = e.x, my[1] = e.y, mh[0] = e.z, mh[1] = e.w;
+                        my = pack2(e.x, e.y), mh = pack2(e.z, e.w);
                     } else {
-                        my[0] = na.emy, my[1] = nb.emy, mh[0] = na.hymy, mh[1] = nb.hymy;
+                        my = na.emy, mh = na.hymy;
                     }
                     if (NOX)
-                        pull_row(in.cur[k], ey, hy, my, mh, false, false, false, ca, cb);
+                        pull_row(in.cur[k], ey, hy, my, mh, false, false, false, c);
                     else
-                        pull_row(in.cur[k], ey, hy, my, mh, xa0, xa_last, xb_last, ca, cb);
+                        pull_row(in.cur[k], ey, hy, my, mh, xa0, xa_last, xb_last, c);
                     idq = in.ids[k];
                 }
-                if (!NOX && src_lane && t + k >= 1) inject_source_t(kind, r.src_g[k], r.src_inc[k], ca);
-                const MatT<float> ma = r.table[idq & 0xffu], mb = r.table[(idq >> 8) & 0xffu];
+                if (!NOX && src_lane && t + k >= 1) {
+                    if (kind == SRC_OPEN) {
+                        c.epx = pack2(__fadd_rn(lo2(c.epx), r.src_g[k]), hi2(c.epx));
+                    } else {
+                        c.epx = pack2(r.src_inc[k], hi2(c.epx));
+                        c.hxpx = pack2(0.f, hi2(c.hxpx));
+                    }
+                }
+                const PairMat mat = pair_mat(r.table[idq & 0xffu], r.table[(idq >> 8) & 0xffu]);
                 const bool owned = out_lane && (FAST || (q >= y0 && q < y1));
                 const bool store = k == BT - 1 && owned;
-                if (F16 && k == BT - 1) {
-                    // the stored state of the last level: fields and FP16 deviations g = f - f^eq
-                    float E3a, Hxa, Hya, Da, E3b, Hxb, Hyb, Db;
-                    moments(ca, ma, &E3a, &Hxa, &Hya, &Da);
-                    moments(cb, mb, &E3b, &Hxb, &Hyb, &Db);
-                    if constexpr (ACC) {  // the fields of the stored level, staged as at the others
-                        if (owned && t + k >= u.acc_from && t + k < u.steps && q >= u.ay0 && q <= u.ay1) {
-                            const float f3a[3] = {Da * ma.inv_eps, Hxa, Hya}, f3b[3] = {Db * mb.inv_eps, Hxb, Hyb};
-                            stage_owned(u.stage, slots[k].x, k, f3a);
-                            if (two) stage_owned(u.stage, slots[k].y, k, f3b);
+                // ACC: a row of contour stencil sites in the accumulated period (uniform over the warp)
+                const bool acc_row = ACC && t + k >= u.acc_from && t + k < u.steps && q >= u.ay0 && q <= u.ay1 &&
+                                     (FAST || (q >= y0 && q < y1));
+                f2 e3, f3[3];
+                if constexpr (F16) {
+                    if (k == BT - 1) {
+                        // the stored state of the last level: fields and FP16 deviations g = f - f^eq
+                        f2 Hx, Hy, d;
+                        moments_pair(c, mat, e3, Hx, Hy, d);
+                        if constexpr (ACC) {  // the fields of the stored level, staged as at the others
+                            if (acc_row && out_lane) {
+                                const f2 f = mul2(d, mat.inv);
+                                stage_owned(u.stage, slots[k].x, k, lo2(f), lo2(Hx), lo2(Hy));
+                                if (two) stage_owned(u.stage, slots[k].y, k, hi2(f), hi2(Hx), hi2(Hy));
+                            }
                         }
-                    }
-                    if (store) {
-                        bad |= field_runaway(E3a, u.runaway) || (two && field_runaway(E3b, u.runaway));
-                        const Fld Fa = stored_fields(E3a, Hxa, Hya), Fb = stored_fields(E3b, Hxb, Hyb);
-                        __half2 g2[NPLANES];
-                        encode_pair(ca, cb, Fa, Fb, u.scale, g2);
-                        const size_t idx = (size_t)q * u.pitch + xa;
-                        if (two) {
+                        if (store) {
+                            bad |= field_runaway(lo2(e3), u.runaway) || (two && field_runaway(hi2(e3), u.runaway));
+                            const f2 third = both(1.0f / 3.0f), n3 = both(-3.0f);
+                            const f2 hx3 = quot2(Hx, n3, third), hy3 = quot2(Hy, n3, third);
+                            __half2 g2[NPLANES];
+                            encode_pair2(c, e3, hx3, hy3, u.scale, g2);
+                            const size_t idx = (size_t)q * u.pitch + xa;
+                            if (two) {
 #pragma unroll
-                            for (int p = 0; p < NPLANES; ++p)
-                                *reinterpret_cast<__half2 *>(u.g_out + p * ps + idx) = g2[p];
-                            *reinterpret_cast<float2 *>(u.fe_out + idx) = make_float2(Fa.e, Fb.e);
-                            *reinterpret_cast<float2 *>(u.fhx_out + idx) = make_float2(Fa.hx, Fb.hx);
-                            *reinterpret_cast<float2 *>(u.fhy_out + idx) = make_float2(Fa.hy, Fb.hy);
-                        } else {
+                                for (int p = 0; p < NPLANES; ++p)
+                                    *reinterpret_cast<__half2 *>(u.g_out + p * ps + idx) = g2[p];
+                            } else {
 #pragma unroll
-                            for (int p = 0; p < NPLANES; ++p) u.g_out[p * ps + idx] = __low2half(g2[p]);
-                            u.fe_out[idx] = Fa.e;
-                            u.fhx_out[idx] = Fa.hx;
-                            u.fhy_out[idx] = Fa.hy;
-                        }
-                    }
-                } else {
-                    bool ra, rb;
-                    if (ACC && t + k >= u.acc_from && t + k < u.steps && q >= u.ay0 && q <= u.ay1 &&
-                        (FAST || (q >= y0 && q < y1))) {
-                        // a row of contour stencil sites in the accumulated period (uniform over the
-                        // warp): the fields of the owned sites enter their Fourier sums
-                        float f3a[3], f3b[3];
-                        ra = update_site_f3<POL>(ca, ma, u.runaway, f3a);
-                        rb = update_site_f3<POL>(cb, mb, u.runaway, f3b);
-                        if (out_lane) {
-                            stage_owned(u.stage, slots[k].x, k, f3a);
-                            if (two) stage_owned(u.stage, slots[k].y, k, f3b);
+                                for (int p = 0; p < NPLANES; ++p) u.g_out[p * ps + idx] = __low2half(g2[p]);
+                            }
+                            store2(u.fe_out + idx, two, e3);
+                            store2(u.fhx_out + idx, two, hx3);
+                            store2(u.fhy_out + idx, two, hy3);
                         }
                     } else {
-                        ra = update_site<POL, true>(ca, ma, u.runaway, nullptr, nullptr);
-                        rb = update_site<POL, true>(cb, mb, u.runaway, nullptr, nullptr);
+                        update_pair<POL, ACC>(c, mat, e3, f3);
+                    }
+                } else {
+                    update_pair<POL, ACC>(c, mat, e3, f3);
+                }
+                if (!(F16 && k == BT - 1)) {
+                    if constexpr (ACC) {  // the fields of the owned sites enter their Fourier sums
+                        if (acc_row && out_lane) {
+                            stage_owned(u.stage, slots[k].x, k, lo2(f3[0]), lo2(f3[1]), lo2(f3[2]));
+                            if (two) stage_owned(u.stage, slots[k].y, k, hi2(f3[0]), hi2(f3[1]), hi2(f3[2]));
+                        }
                     }
                     if (store) {
-                        bad |= ra || (two && rb);
+                        bad |= field_runaway(lo2(e3), u.runaway) || (two && field_runaway(hi2(e3), u.runaway));
                         float *f = u.fout + (size_t)q * u.pitch + xa;
-                        store2(f + P_EZ * ps, two, ca.ez, cb.ez);
-                        store2(f + P_EPX * ps, two, ca.epx, cb.epx);
-                        store2(f + P_EMX * ps, two, ca.emx, cb.emx);
-                        store2(f + P_EPY * ps, two, ca.epy, cb.epy);
-                        store2(f + P_EMY * ps, two, ca.emy, cb.emy);
-                        store2(f + P_HXPX * ps, two, ca.hxpx, cb.hxpx);
-                        store2(f + P_HXMX * ps, two, ca.hxmx, cb.hxmx);
-                        store2(f + P_HXZ * ps, two, ca.hxz, cb.hxz);
-                        store2(f + P_HYPY * ps, two, ca.hypy, cb.hypy);
-                        store2(f + P_HYMY * ps, two, ca.hymy, cb.hymy);
-                        store2(f + P_HYZ * ps, two, ca.hyz, cb.hyz);
+                        store2(f + P_EZ * ps, two, c.ez);
+                        store2(f + P_EPX * ps, two, c.epx);
+                        store2(f + P_EMX * ps, two, c.emx);
+                        store2(f + P_EPY * ps, two, c.epy);
+                        store2(f + P_EMY * ps, two, c.emy);
+                        store2(f + P_HXPX * ps, two, c.hxpx);
+                        store2(f + P_HXMX * ps, two, c.hxmx);
+                        store2(f + P_HXZ * ps, two, c.hxz);
+                        store2(f + P_HYPY * ps, two, c.hypy);
+                        store2(f + P_HYMY * ps, two, c.hymy);
+                        store2(f + P_HYZ * ps, two, c.hyz);
                     }
                 }
             }
@@ -585,14 +558,14 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
             } else {
                 // level k moves on by one row: row i - k becomes the kept row
                 if (FAST || have) {
-                    if (!FAST && i - k == ny - 1) edge[k * 32 + lane] = make_float4(na.emy, nb.emy, na.hymy, nb.hymy);
-                    out.oe[k][0] = in.cur[k].epy[0], out.oe[k][1] = in.cur[k].epy[1];
-                    out.oh[k][0] = in.cur[k].hypy[0], out.oh[k][1] = in.cur[k].hypy[1];
-                    keep_row(out.cur[k], na, nb);
+                    if (!FAST && i - k == ny - 1)
+                        edge[k * 32 + lane] = make_float4(lo2(na.emy), hi2(na.emy), lo2(na.hymy), hi2(na.hymy));
+                    out.oe[k] = in.cur[k].epy;
+                    out.oh[k] = in.cur[k].hypy;
+                    keep_row(out.cur[k], na);
                 }
             }
-            na = ca;
-            nb = cb;
+            na = c;
             have = compute;
         }
         // ids: row i - 1 - k for level k + 1 at the next row
