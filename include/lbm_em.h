@@ -373,7 +373,10 @@ typedef struct {
                                 instance through four time levels held in registers (the
                                 autotuner picks the segment height, 64, 128 or 256 rows); same
                                 bits as one step per launch.  2: the TMA tile kernel above.  With 0 the
-                                autotuner times every kind that applies                    */
+                                autotuner times every kind that applies; with conv_tol > 0
+                                (FP32, nothing pinned) that is the four-step kernel for the
+                                steps between the period boundaries and the one-step kernel
+                                at them, unless many different periods leave few such gaps  */
 } lbm_em_batch_opts;
 
 typedef struct lbm_em_batch lbm_em_batch_t;

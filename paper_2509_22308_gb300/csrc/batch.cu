@@ -224,8 +224,7 @@ __device__ __forceinline__ void batch_acc(const double *f3, const int *slot, dou
 // copies of its next tile as soon as phase 1 has read the stage.  The per-site arithmetic
 // is the one-step kernel's (same bits).  An instance whose run ends at t + 1 takes only
 // the first step (its state is not needed afterwards; its forces come from the
-// accumulators).  Convergence exits need a decision between any two steps, so they keep
-// the one-step kernel.
+// accumulators).
 // ACC: the tile's instance accumulates at t or t + 1; without it no FP64 operation is
 // compiled in (a run-time accumulation test per site let the compiler predicate the FP64
 // conversions of the field triple into every site's update, and GB300's FP64 pipe made
@@ -394,8 +393,9 @@ __global__ void __launch_bounds__(NTH, 3)
 // After a step of time t (*t_next = t + 1): every instance at a period boundary compares
 // its energy with the previous boundary's (Sec. III convergence criterion); once two
 // successive changes are <= tol * W and at least min_periods - 1 periods have run, the
-// instance runs one more period, with Fourier accumulation, and stops.
-__global__ void k_batch_converge(InstDesc *desc, double *energy, double *prev, int *settled,
+// instance runs one more period, with Fourier accumulation, and stops.  si: the four-step kernel's
+// records, which hold the run lengths too (NULL without them).
+__global__ void k_batch_converge(InstDesc *desc, StreamInst *si, double *energy, double *prev, int *settled,
                                  const long long *__restrict__ t_next, double tol, int min_periods, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -412,6 +412,10 @@ __global__ void k_batch_converge(InstDesc *desc, double *energy, double *prev, i
     if (s >= 2 && periods_done + 1 >= min_periods) {
         d.acc_from = t + 1;
         d.steps = t + 1 + d.period;
+        if (si) {
+            si[i].acc_from = d.acc_from;
+            si[i].steps = d.steps;
+        }
     }
 }
 
@@ -510,13 +514,14 @@ struct lbm_em_batch {
     int four_seg = 0, four_grid = 0, four_blocks = 0, four_ctas = 0, n_units = 0;
     int4 *d_units = nullptr;
     StreamInst *d_sinsts = nullptr;
+    std::vector<StreamInst> sinsts;  // host copy, restored when a run starts (convergence exits change run lengths)
     SourceParams *d_srcp = nullptr;
     SrcLevels *d_srcs4 = nullptr;
     CUtensorMap *d_smaps4 = nullptr;
     float *d_stage4 = nullptr;  // staged stencil fields of the accumulating launches (12 per slot)
     int *d_slot_inst = nullptr; // each accumulator slot's instance
     int want_spl = 0;  // lbm_em_batch_opts.steps_per_launch
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // two launches, starting with the state in buf[0], buf[1]
     bool ran = false;
     // a bounded wait for a tile copy gave up (seen by lbm_em_batch_results): a copy may
     // still have been in flight when its CTA left, so the batch refuses further runs
@@ -524,6 +529,7 @@ struct lbm_em_batch {
     // convergence exits
     double conv_tol = 0.0;
     int min_periods = 1;
+    std::vector<std::pair<int, long long>> periods;  // distinct periods and the longest run of each
     double *d_energy = nullptr, *d_prev = nullptr;
     int *d_settled = nullptr;
 };
@@ -532,7 +538,8 @@ static void batch_free(lbm_em_batch *b) {
     if (!b) return;
     cudaSetDevice(b->dev);
     if (b->stream) cudaStreamSynchronize(b->stream);
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    for (cudaGraphExec_t g : b->graph)
+        if (g) cudaGraphExecDestroy(g);
     dfree(b->buf[0]);
     dfree(b->buf[1]);
     dfree(b->d_mat);
@@ -611,7 +618,8 @@ static lbm_em_status batch_tiles(lbm_em_batch *b, int tw, int th) {
 // columns in L2); and the per-instance records with that segment height.
 static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
     std::vector<int4> units;
-    std::vector<StreamInst> si(b->n);
+    std::vector<StreamInst> &si = b->sinsts;
+    si.resize(b->n);
     for (int i = 0; i < b->n; ++i) {
         const InstDesc &d = b->desc[i];
         StreamInst &r = si[i];
@@ -729,8 +737,8 @@ static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p) {
             k_batch_step<float, POL_TM><<<grid, 256, 0, s>>>(a, b->d_time + p, b->d_time + (1 - p));
     }
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && b->conv_tol > 0.0) {
-        k_batch_converge<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->d_energy, b->d_prev, b->d_settled,
+    if (e == cudaSuccess && b->conv_tol > 0.0 && !b->four) {  // (no period boundary inside a four-step launch)
+        k_batch_converge<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->d_sinsts, b->d_energy, b->d_prev, b->d_settled,
                                                            b->d_time + (1 - p), b->conv_tol, b->min_periods, b->n);
         e = cudaGetLastError();
     }
@@ -751,6 +759,51 @@ static cudaError_t batch_launch_one(lbm_em_batch *b, cudaStream_t s, int p) {
 // Steps one launch of the batch's configuration advances.
 static int batch_spl(const lbm_em_batch *b) { return b->four ? 4 : b->two ? 2 : 1; }
 
+// Convergence exits: the steps from time t to the next time where a one-step launch has to begin
+// or end.  An instance's energy is sampled by the step at a multiple of its period (> 0), which
+// the one-step kernel takes and k_batch_converge follows; its accumulated period and its run begin
+// and end there or one step later.  So between these times any launch may take several steps.
+static long long conv_gap(const lbm_em_batch *b, long long t) {
+    long long gap = b->max_steps - t;
+    for (const auto &p : b->periods) {
+        if (t >= p.second) continue;  // every instance of this period has ended
+        const long long r = t % p.first;
+        gap = std::min(gap, r == 0 && t > 0 ? 1 : p.first - r);
+    }
+    return gap;
+}
+
+// Whether four-step launches take at least half of a convergence run's steps.  With one period P they
+// take all but one to four steps of each (180 against 57 GLUPS on 96 instances of 200^2); with many
+// different periods in one batch few gaps hold four steps, and the one-step kernel on its tuned
+// tiles is as good.
+static bool conv_four(const lbm_em_batch *b) {
+    long long in4 = 0;
+    for (long long t = 0; t < b->max_steps;) {
+        const long long gap = conv_gap(b, t);
+        in4 += gap / 4 * 4;
+        t += gap;
+    }
+    return 2 * in4 >= b->max_steps;
+}
+
+// The graph of two launches that starts with the state in buf[p].
+static lbm_em_status batch_capture(lbm_em_batch *b, int p) {
+    cudaGraph_t g = nullptr;
+    lbm_em_status st = cuda_status(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
+    if (st) return st;
+    cudaError_t e = batch_launch(b, b->cap, p);
+    if (e == cudaSuccess) e = batch_launch(b, b->cap, 1 - p);
+    cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
+    if (e != cudaSuccess || e2 != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return cuda_status(e != cudaSuccess ? e : e2, "capturing the batch graph");
+    }
+    e = cudaGraphInstantiate(&b->graph[p], g, 0);
+    cudaGraphDestroy(g);
+    return cuda_status(e, "cudaGraphInstantiate");
+}
+
 static lbm_em_status batch_clear(lbm_em_batch *b) {
     lbm_em_status st = cuda_status(cudaMemsetAsync(b->buf[0], 0, b->buf_elems * b->elem, b->stream), "clear");
     if (!st) st = cuda_status(cudaMemsetAsync(b->d_acc, 0, b->acc_slots * 6 * sizeof(double), b->stream), "clear");
@@ -764,15 +817,19 @@ static lbm_em_status batch_clear(lbm_em_batch *b) {
         st = cuda_status(copy_async(b->d_desc, b->desc.data(), b->n * sizeof(InstDesc), cudaMemcpyHostToDevice,
                                          b->stream),
                          "restoring descriptors");
+    if (!st && b->four && b->conv_tol > 0.0)
+        st = cuda_status(copy_async(b->d_sinsts, b->sinsts.data(), b->n * sizeof(StreamInst), cudaMemcpyHostToDevice,
+                                    b->stream),
+                         "restoring stream records");
     if (!st) st = cuda_status(cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
     return st;
 }
 
 // Time a few steps of each (tile shape, CTAs per SM, steps per launch) candidate from the
 // cleared state.  FP32 runs of fixed length also have the two-step kernel (TMA-staged 64 x 8,
-// 32 x 16 and 40 x 12 tiles, as many CTAs per SM as their shared memory allows) and the
-// four-step row-streaming kernel (row segments of 64, 128 or 256 rows; its runs end with
-// one-step launches on 64 x 4 tiles).  lbm_em_batch_opts.steps_per_launch restricts the
+// 32 x 16 and 40 x 12 tiles, as many CTAs per SM as their shared memory allows); these and most FP32
+// runs with convergence exits (conv_four) have the four-step row-streaming kernel (row segments of
+// 64, 128 or 256 rows; the steps that it cannot take are one-step launches on 64 x 4 tiles).  lbm_em_batch_opts.steps_per_launch restricts the
 // candidates to one kind; a pinned tile shape or CTA count to the matching ones.
 static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int want_c) {
     struct Cand {
@@ -781,7 +838,7 @@ static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int
     std::vector<Cand> cands;
     const bool pinned = want_w || want_h || want_c;
     const bool multi = b->prec == LBM_EM_F32 && b->conv_tol <= 0.0;
-    if (multi && b->four_grid > 0 && ((b->want_spl == 0 && !pinned) || b->want_spl == 4))
+    if ((multi || (b->prec == LBM_EM_F32 && conv_four(b))) && b->four_grid > 0 && ((b->want_spl == 0 && !pinned) || b->want_spl == 4))
         for (int seg : {64, 128, 256}) cands.push_back(Cand{64, 4, 4, 4, seg});
     const int two_shapes[3][2] = {{GeoWide::KW, GeoWide::KH}, {GeoTall::KW, GeoTall::KH}, {GeoMid::KW, GeoMid::KH}};
     for (int g = 0; g < 3; ++g) {
@@ -920,6 +977,7 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
     std::map<int, size_t> cs_at;    // period -> offset of its phase table in cs_all
     std::vector<double2> cs_all;
     std::vector<size_t> cs_off(n);
+    std::map<int, long long> run_of;  // period -> longest run
     b->desc.resize(n);
     size_t base = 0, mat = 0, slot = 0, accs = 0;
     for (int i = 0; i < n; ++i) {
@@ -940,6 +998,8 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
         d.steps = (long long)s.periods * s.period_steps;
         d.acc_from = d.steps - s.period_steps;
         b->max_steps = std::max(b->max_steps, d.steps);
+        long long &longest = run_of[d.period];
+        longest = std::max(longest, d.steps);
         lbm_em_contour c{std::nan(""), std::nan(""), s.contour_radius, s.n_points, 0, s.janus.a};
         if (!std::isnan(s.janus.cx)) c.cx = s.janus.cx;
         if (!std::isnan(s.janus.cy)) c.cy = s.janus.cy;
@@ -996,6 +1056,7 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
             }
         }
     }
+    b->periods.assign(run_of.begin(), run_of.end());
     b->buf_elems = base;
     b->mat_bytes = mat;
     b->slot_elems = slot;
@@ -1079,7 +1140,7 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
         BTRY(dmalloc(&b->d_srcs, (size_t)n * sizeof(SrcPairF)), "cudaMalloc(source values)");
         // the four-step kernel: per instance the three tensor maps of its rows, its source
         // parameters, room for a launch's source values
-        if (o->conv_tol <= 0.0 && (o->steps_per_launch == 0 || o->steps_per_launch == 4)) {
+        if (o->steps_per_launch == 0 || o->steps_per_launch == 4) {
             int warps = 0;
             BTRY(batch_stream_prepare(&warps), "configuring the four-step batch kernel");
             b->four_grid = warps / kStreamWarps;  // resident blocks (reported per SM)
@@ -1151,43 +1212,36 @@ lbm_em_status lbm_em_batch_run(lbm_em_batch_t *b) {
     lbm_em_status st = batch_clear(b);
     if (!st) st = cuda_status(batch_rasterize(b), "rasterise");
     if (st) return st;
-    if (!b->graph) {
-        cudaGraph_t g = nullptr;
-        st = cuda_status(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
-        if (st) return st;
-        cudaError_t e = batch_launch(b, b->cap, 0);
-        if (e == cudaSuccess) e = batch_launch(b, b->cap, 1);
-        cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
-        if (e != cudaSuccess || e2 != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            return cuda_status(e != cudaSuccess ? e : e2, "capturing the batch graph");
-        }
-        e = cudaGraphInstantiate(&b->graph, g, 0);
-        cudaGraphDestroy(g);
-        st = cuda_status(e, "cudaGraphInstantiate");
-        if (st) return st;
-    }
-    // the graph holds two launches (state buf[0] -> buf[1] -> buf[0]) of spl steps each; the
-    // tail runs at most one more multi-step launch and then one-step launches
+    // a graph holds two launches (state buf[p] -> buf[1 - p] -> buf[p]) of spl steps each; the
+    // steps that are left at the end, or (four steps per launch with convergence exits) before a
+    // time that a one-step launch has to begin or end at, take at most one more multi-step launch
+    // and then one-step launches
     const long long spl = batch_spl(b), per_graph = 2 * spl;
+    const bool stops = b->four && b->conv_tol > 0.0;
     long long t = 0;
     int p = 0;
-    while (t + per_graph <= b->max_steps) {
-        st = cuda_status(cudaGraphLaunch(b->graph, b->stream), "cudaGraphLaunch");
-        if (st) return st;
-        t += per_graph;
-    }
-    if (spl > 1 && t + spl <= b->max_steps) {
-        st = cuda_status(batch_launch(b, b->stream, p), "batch step");
-        if (st) return st;
-        p ^= 1;
-        t += spl;
-    }
     while (t < b->max_steps) {
-        st = cuda_status(batch_launch_one(b, b->stream, p), "batch step");
-        if (st) return st;
-        p ^= 1;
-        ++t;
+        long long left = stops ? conv_gap(b, t) : b->max_steps - t;
+        t += left;
+        if (left >= per_graph && !b->graph[p]) {
+            st = batch_capture(b, p);
+            if (st) return st;
+        }
+        for (; left >= per_graph; left -= per_graph) {
+            st = cuda_status(cudaGraphLaunch(b->graph[p], b->stream), "cudaGraphLaunch");
+            if (st) return st;
+        }
+        if (spl > 1 && left >= spl) {
+            st = cuda_status(batch_launch(b, b->stream, p), "batch step");
+            if (st) return st;
+            p ^= 1;
+            left -= spl;
+        }
+        for (; left > 0; --left) {
+            st = cuda_status(batch_launch_one(b, b->stream, p), "batch step");
+            if (st) return st;
+            p ^= 1;
+        }
     }
     k_batch_contour<<<b->n, 256, 0, b->stream>>>(b->d_cdesc, b->d_pts, b->d_acc, b->d_out);
     st = cuda_status(cudaGetLastError(), "batch contour");
