@@ -16,6 +16,7 @@
 // each candidate on the actual packed data (then the state is cleared).
 #include <algorithm>
 #include <array>
+#include <climits>
 #include <type_traits>
 #include <cmath>
 #include <cstring>
@@ -508,7 +509,7 @@ struct lbm_em_batch {
     SrcPairF *d_srcs = nullptr;     // FP32: per instance, the source values of the current launch
     int two_ctas[3] = {0, 0, 0};
     // four steps per launch (FP32, fixed run lengths): row-streaming kernel over work units
-    // (instance, strip, row segment of four_seg rows), per-instance records, tensor maps and
+    // (instance, strip, row segment of at most four_seg rows), per-instance records, tensor maps and
     // source parameters, and the source values of the current launch
     bool four = false;
     int four_seg = 0, four_grid = 0, four_blocks = 0, four_ctas = 0, n_units = 0;
@@ -516,12 +517,12 @@ struct lbm_em_batch {
     StreamInst *d_sinsts = nullptr;
     std::vector<StreamInst> sinsts;  // host copy, restored when a run starts (convergence exits change run lengths)
     SourceParams *d_srcp = nullptr;
-    SrcLevels *d_srcs4 = nullptr;
     CUtensorMap *d_smaps4 = nullptr;
     float *d_stage4 = nullptr;  // staged stencil fields of the accumulating launches (12 per slot)
     int *d_slot_inst = nullptr; // each accumulator slot's instance
     int want_spl = 0;  // lbm_em_batch_opts.steps_per_launch
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // two launches, starting with the state in buf[0], buf[1]
+    cudaGraphExec_t graph[2][3] = {};  // two launches that start with the state in buf[p], by StepKind
+    long long first_acc = 0, last_plain = 0;  // see batch_kind
     bool ran = false;
     // a bounded wait for a tile copy gave up (seen by lbm_em_batch_results): a copy may
     // still have been in flight when its CTA left, so the batch refuses further runs
@@ -538,8 +539,9 @@ static void batch_free(lbm_em_batch *b) {
     if (!b) return;
     cudaSetDevice(b->dev);
     if (b->stream) cudaStreamSynchronize(b->stream);
-    for (cudaGraphExec_t g : b->graph)
-        if (g) cudaGraphExecDestroy(g);
+    for (auto &of_buf : b->graph)
+        for (cudaGraphExec_t g : of_buf)
+            if (g) cudaGraphExecDestroy(g);
     dfree(b->buf[0]);
     dfree(b->buf[1]);
     dfree(b->d_mat);
@@ -562,7 +564,6 @@ static void batch_free(lbm_em_batch *b) {
     dfree(b->d_units);
     dfree(b->d_sinsts);
     dfree(b->d_srcp);
-    dfree(b->d_srcs4);
     dfree(b->d_smaps4);
     dfree(b->d_stage4);
     dfree(b->d_slot_inst);
@@ -613,7 +614,14 @@ static lbm_em_status batch_tiles(lbm_em_batch *b, int tw, int th) {
     return st;
 }
 
-// The four-step kernel's work units for row segments of `seg` rows: instance by decreasing run
+// The height of equal row segments of at most `seg` rows: the fewest segments, and none much shorter than
+// the others (200 rows by 64: 4 x 50, not 3 x 64 + 8), so that no unit lasts longer than it must.
+static int even_rows(int ny, int seg) {
+    const int segs = (ny + seg - 1) / seg;
+    return (ny + segs - 1) / segs;
+}
+
+// The four-step kernel's work units for row segments of at most `seg` rows: instance by decreasing run
 // length, then segment, then strip (neighbouring strips run side by side and share their halo
 // columns in L2); and the per-instance records with that segment height.
 static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
@@ -625,7 +633,7 @@ static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
         StreamInst &r = si[i];
         std::memset(&r, 0, sizeof(r));
         r.nx = d.nx, r.ny = d.ny, r.pitch = d.pitch, r.kind = d.src.kind;
-        r.seg_rows = seg, r.n_strips = (d.nx + kStreamOutW - 1) / kStreamOutW, r.ay0 = d.y0, r.ay1 = d.y1;
+        r.seg_rows = even_rows(d.ny, seg), r.n_strips = (d.nx + kStreamOutW - 1) / kStreamOutW, r.ay0 = d.y0, r.ay1 = d.y1;
         r.steps = d.steps, r.acc_from = d.acc_from, r.base = (long long)d.base, r.pstride = (long long)d.pstride;
         r.slot_base = (long long)d.slot_base, r.acc_base = d.acc_base, r.period = d.period;
         r.cs = d.src.cs;
@@ -634,8 +642,8 @@ static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
     }
     for (long long ii : b->order) {
         const int i = (int)ii;
-        for (int y = 0; y < b->desc[i].ny; y += seg)
-            for (int st = 0; st < si[i].n_strips; ++st) units.push_back(make_int4(i, st, y / seg, 0));
+        for (int y = 0; y < b->desc[i].ny; y += si[i].seg_rows)
+            for (int st = 0; st < si[i].n_strips; ++st) units.push_back(make_int4(i, st, y / si[i].seg_rows, 0));
     }
     dfree(b->d_units);
     b->d_units = nullptr;
@@ -695,9 +703,12 @@ static void launch_batch_step2(const lbm_em_batch *b, const BatchArgs<float> &a,
                                                                          b->d_time + p, b->d_time + (1 - p));
 }
 
-// One launch from the state in buf[p] (time word p) to buf[1 - p]: one step, or two with
-// b->two.  The caller alternates p launch by launch.
-static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p) {
+// Which instances a four-step launch can find (batch_kind).
+enum StepKind { kPlainOnly, kBoth, kAccOnly };
+
+// One launch from the state in buf[p] (time word p) to buf[1 - p]: one step, two with b->two,
+// four with b->four (kind: of the instances it finds).  The caller alternates p launch by launch.
+static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, StepKind kind = kBoth) {
     const int grid = b->ctas * b->sms;
     if (b->prec == LBM_EM_F32X2) {
         BatchArgs<df> a{b->d_desc, b->d_tiles, b->n_tiles, b->tile_w, b->tile_h, ilog2(b->tile_w),
@@ -720,10 +731,10 @@ static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p) {
                            (const float *)b->buf[p], (float *)b->buf[1 - p], b->d_mat, b->d_slot,
                            b->d_acc, b->d_err, b->d_energy, b->conv_tol > 0.0};
         if (b->four) {
-            launch_batch_step4(b->d_sinsts, b->d_srcp, b->n, b->d_units, b->n_units, b->d_srcs4, b->d_smaps4, p,
+            launch_batch_step4(b->d_sinsts, b->d_srcp, b->d_units, b->n_units, b->d_smaps4, p,
                                (float *)b->buf[1 - p], b->d_slot, b->d_acc, b->d_stage4, b->d_slot_inst,
                                (int)b->acc_slots, b->d_err, b->d_time + p, b->d_time + (1 - p), b->four_blocks,
-                               b->pol, s);
+                               b->pol, kind != kAccOnly, kind != kPlainOnly, s);
         } else if (b->two) {
             k_batch_source<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->n, b->d_time + p, b->d_srcs);
             if (b->pol == POL_TE)
@@ -787,19 +798,28 @@ static bool conv_four(const lbm_em_batch *b) {
     return 2 * in4 >= b->max_steps;
 }
 
+// The instances that `n` four-step launches from time t can find.  first_acc: the earliest time that an
+// accumulated period can begin at; last_plain: the latest.  With convergence exits that is
+// decided on the device, but never before the third sample (k_batch_converge compares two
+// changes) or min_periods, and never after the nominal time.
+static StepKind batch_kind(const lbm_em_batch *b, long long t, int n) {
+    if (t + 4 * n - 1 < b->first_acc) return kPlainOnly;
+    return t + 3 >= b->last_plain ? kAccOnly : kBoth;
+}
+
 // The graph of two launches that starts with the state in buf[p].
-static lbm_em_status batch_capture(lbm_em_batch *b, int p) {
+static lbm_em_status batch_capture(lbm_em_batch *b, int p, StepKind kind) {
     cudaGraph_t g = nullptr;
     lbm_em_status st = cuda_status(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
     if (st) return st;
-    cudaError_t e = batch_launch(b, b->cap, p);
-    if (e == cudaSuccess) e = batch_launch(b, b->cap, 1 - p);
+    cudaError_t e = batch_launch(b, b->cap, p, kind);
+    if (e == cudaSuccess) e = batch_launch(b, b->cap, 1 - p, kind);
     cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return cuda_status(e != cudaSuccess ? e : e2, "capturing the batch graph");
     }
-    e = cudaGraphInstantiate(&b->graph[p], g, 0);
+    e = cudaGraphInstantiate(&b->graph[p][kind], g, 0);
     cudaGraphDestroy(g);
     return cuda_status(e, "cudaGraphInstantiate");
 }
@@ -1057,6 +1077,12 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
         }
     }
     b->periods.assign(run_of.begin(), run_of.end());
+    b->first_acc = LLONG_MAX;
+    for (const InstDesc &d : b->desc) {
+        const long long exit = o->conv_tol > 0.0 ? (long long)std::max(3, o->min_periods - 1) * d.period + 1 : LLONG_MAX;
+        b->first_acc = std::min(b->first_acc, std::min(d.acc_from, exit));
+        b->last_plain = std::max(b->last_plain, d.acc_from);
+    }
     b->buf_elems = base;
     b->mat_bytes = mat;
     b->slot_elems = slot;
@@ -1167,7 +1193,6 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
             BTRY(dmalloc(&b->d_srcp, (size_t)n * sizeof(SourceParams)), "cudaMalloc(source parameters)");
             BTRY(copy_async(b->d_srcp, sp.data(), sp.size() * sizeof(SourceParams), cudaMemcpyHostToDevice, b->stream),
                  "upload");
-            BTRY(dmalloc(&b->d_srcs4, (size_t)n * sizeof(SrcLevels)), "cudaMalloc(source values)");
             // the accumulating launches' staged fields (12 floats per stencil slot) and each
             // slot's instance, for the flush that adds them to the Fourier sums
             if (accs > 0) {
@@ -1222,21 +1247,23 @@ lbm_em_status lbm_em_batch_run(lbm_em_batch_t *b) {
     int p = 0;
     while (t < b->max_steps) {
         long long left = stops ? conv_gap(b, t) : b->max_steps - t;
-        t += left;
-        if (left >= per_graph && !b->graph[p]) {
-            st = batch_capture(b, p);
-            if (st) return st;
-        }
-        for (; left >= per_graph; left -= per_graph) {
-            st = cuda_status(cudaGraphLaunch(b->graph[p], b->stream), "cudaGraphLaunch");
+        for (; left >= per_graph; left -= per_graph, t += per_graph) {
+            const StepKind kind = b->four ? batch_kind(b, t, 2) : kBoth;
+            if (!b->graph[p][kind]) {
+                st = batch_capture(b, p, kind);
+                if (st) return st;
+            }
+            st = cuda_status(cudaGraphLaunch(b->graph[p][kind], b->stream), "cudaGraphLaunch");
             if (st) return st;
         }
         if (spl > 1 && left >= spl) {
-            st = cuda_status(batch_launch(b, b->stream, p), "batch step");
+            st = cuda_status(batch_launch(b, b->stream, p, b->four ? batch_kind(b, t, 1) : kBoth), "batch step");
             if (st) return st;
             p ^= 1;
             left -= spl;
+            t += spl;
         }
+        t += left;
         for (; left > 0; --left) {
             st = cuda_status(batch_launch_one(b, b->stream, p), "batch step");
             if (st) return st;

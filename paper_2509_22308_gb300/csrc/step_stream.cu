@@ -85,20 +85,20 @@ struct Layout {
 static_assert(3 * (Layout<false>::SMEM + 1024 + 256) <= 233472 && 3 * (Layout<true>::SMEM + 1024 + 256) <= 233472,
               "three blocks per SM");
 
-// Not inlined, called by one thread: see source_pair_f.
-static __device__ __noinline__ SrcLevels source_levels_f(const SourceParams src, long long t) {
-    SrcLevels v;
-    for (int k = 0; k < BT; ++k) v.g[k] = v.inc[k] = 0.f;
-    if (src.kind != SRC_NONE) {
-        for (int k = 0; k < BT; ++k) {
-            if (t + k < 1) continue;
-            double g, inc;
-            source_values(src, t + k, &g, &inc);
-            v.g[k] = (float)g;
-            v.inc[k] = (float)inc;
-        }
+// The source values of the launch's four times, one time per lane (lanes 0 .. 3), by a warp whose strip
+// holds column 0, before it starts.  No other warp needs them: evaluated by one thread ahead of the
+// block's barrier (FP64: a division, a sine and a 64-bit remainder per time) they kept every warp
+// waiting for a tenth of the launch, and as a kernel of its own ahead of the batch's launch they
+// cost its latency.  Not inlined: see source_pair_f.
+static __device__ __noinline__ void source_levels_f(const SourceParams src, long long t, SrcLevels *v) {
+    const int k = (int)threadIdx.x & 31;
+    if (k < BT) {
+        double g = 0.0, inc = 0.0;
+        if (t + k >= 1) source_values(src, t + k, &g, &inc);
+        v->g[k] = (float)g;
+        v->inc[k] = (float)inc;
     }
-    return v;
+    __syncwarp();
 }
 
 // The nine populations of a row that the next level reads at the row itself or from its x
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     constexpr int RING = LY::RING;
     extern __shared__ unsigned char sm_dyn[];
     __shared__ __align__(8) uint64_t bars[NW][RING];
-    __shared__ SrcLevels sp;
+    __shared__ SrcLevels sp[NW];
     unsigned char *s = sm_dyn + ((128u - (smem_u32(sm_dyn) & 127u)) & 127u);
     MatT<float> *table = reinterpret_cast<MatT<float> *>(s);
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
@@ -653,7 +653,6 @@ __global__ void __launch_bounds__(NW * 32, 3)
 
     const long long t = *t_in;
     if (blockIdx.x == 0 && threadIdx.x == 0) *t_out = t + BT;
-    if (threadIdx.x == 0) sp = source_levels_f(a.src, t);
     for (int k = threadIdx.x; k < 256; k += NW * 32) table[k] = a.mtab[k];
     if (lane == 0) {
         for (int j = 0; j < RING; ++j) mbar_init(&bars[warp][j], 1);
@@ -663,6 +662,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     const int unit = (int)blockIdx.x * NW + warp;
     if (unit >= a.n_units) return;
     const int strip = unit % a.n_strips, seg = unit / a.n_strips;
+    if (strip == 0 && u.kind != SRC_NONE) source_levels_f(a.src, t, &sp[warp]);
     UnitRun r;
     r.xs = strip * OUTW - HALO;
     r.y0 = seg * a.seg_rows;
@@ -672,8 +672,8 @@ __global__ void __launch_bounds__(NW * 32, 3)
     r.fmap = &fmap;
     r.imap = &imap;
     r.table = table;
-    r.src_g = sp.g;
-    r.src_inc = sp.inc;
+    r.src_g = sp[warp].g;
+    r.src_inc = sp[warp].inc;
     RingState R{ring, bars[warp], reinterpret_cast<float4 *>(ring + RING * LY::SLOT), 0, 0u};
     bool bad = false;
     const bool ok = stream_unit<F16, POL, ACC, !ACC, MIX>(u, r, R, bad);
@@ -684,8 +684,8 @@ __global__ void __launch_bounds__(NW * 32, 3)
 // Batched design maps: the warps walk the work units of every instance (instance, strip, row
 // segment; ordered by decreasing run length, then segment, then strip) with a grid stride,
 // skipping instances that have finished, four steps per launch; the batch launches one warp per
-// unit, so each warp normally takes one.  Two instantiations run one after the other in
-// every launch and split the unfinished instances between them: ACC = false takes those with
+// unit, so each warp normally takes one.  Two instantiations split the unfinished instances between
+// them, one after the other where a launch can have both kinds (launch_batch_step4): ACC = false takes those with
 // no time of their accumulated (last) period among the launch's four, ACC = true the others,
 // whose stencil sites' fields it stages for the levels whose time falls in that period
 // (k_batch_flush4 adds them to the Fourier sums after it; ACC = true takes the general row
@@ -694,7 +694,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
 template <int POL, bool ACC>
 __global__ void __launch_bounds__(NW * 32, 3)
     k_batch_step4(const StreamInst *__restrict__ insts, const int4 *__restrict__ units, int n_units,
-                  const SrcLevels *__restrict__ srcs, const CUtensorMap *__restrict__ maps, int p,
+                  const SourceParams *__restrict__ srcp, const CUtensorMap *__restrict__ maps, int p,
                   float *__restrict__ buf_out, const int *__restrict__ slot, float *__restrict__ stage,
                   unsigned *__restrict__ err, const long long *__restrict__ t_in, long long *__restrict__ t_out) {
     using LY = Layout<false>;
@@ -704,6 +704,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     __shared__ MatT<float> wtab[NW][4];  // the current unit's region table, per warp
     __shared__ UnitCtx uctx[NW];         // the current instance, per warp (read from here, not kept in registers)
     __shared__ UnitRun urun[NW];         // the current unit, per warp
+    __shared__ SrcLevels sp[NW];         // its source values (first strip), per warp
     unsigned char *s = sm_dyn + ((128u - (smem_u32(sm_dyn) & 127u)) & 127u);
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
     unsigned char *ring = s + LY::TABLE + (size_t)warp * LY::WARP;
@@ -753,9 +754,10 @@ __global__ void __launch_bounds__(NW * 32, 3)
             tmap_acquire(r.smap);  // lane 0 issues every row copy of the unit
             tmap_acquire(r.imap);
             r.table = wtab[warp];
-            r.src_g = srcs[un.x].g;
-            r.src_inc = srcs[un.x].inc;
+            r.src_g = sp[warp].g;
+            r.src_inc = sp[warp].inc;
         }
+        if (un.y == 0 && I.kind != SRC_NONE) source_levels_f(srcp[un.x], t, &sp[warp]);
         __syncwarp();
         bool bad = false;
         const bool ok = stream_unit<false, POL, ACC, !ACC>(u, r, R, bad);
@@ -765,13 +767,6 @@ __global__ void __launch_bounds__(NW * 32, 3)
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(err + un.x, kErrUnstable);
     }
-}
-
-// The source values of every instance at the launch's four times, one thread per instance.
-__global__ void k_batch_source4(const SourceParams *__restrict__ src, int n, const long long *__restrict__ t_in,
-                                SrcLevels *__restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = source_levels_f(src[i], *t_in);
 }
 
 // After an accumulating launch from time *t_in: adds every stencil slot's staged FP32 fields of
@@ -955,27 +950,30 @@ cudaError_t encode_batch_stream_maps(CUtensorMap *maps, const float *buf0, const
     return e;
 }
 
-cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, int n_inst, const int4 *units,
-                               int n_units, SrcLevels *srcs, const CUtensorMap *maps, int p, float *buf_out,
-                               const int *slot, double *acc, float *stage, const int *slot_inst, int n_slots,
-                               unsigned *err, const long long *t_in, long long *t_out, int grid, int pol,
-                               cudaStream_t s) {
-    k_batch_source4<<<(n_inst + 127) / 128, 128, 0, s>>>(srcp, n_inst, t_in, srcs);
+cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, const int4 *units, int n_units,
+                               const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
+                               float *stage, const int *slot_inst, int n_slots, unsigned *err, const long long *t_in,
+                               long long *t_out, int grid, int pol, bool plain, bool accumulate, cudaStream_t s) {
     const size_t sm = Layout<false>::SMEM;
     // both write t + 4 to t_out; neither reads it
-    if (pol == POL_TE) {
-        k_batch_step4<POL_TE, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcs, maps, p, buf_out, slot,
-                                                              stage, err, t_in, t_out);
-        k_batch_step4<POL_TE, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcs, maps, p, buf_out, slot,
-                                                             stage, err, t_in, t_out);
-    } else {
-        k_batch_step4<POL_TM, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcs, maps, p, buf_out, slot,
-                                                              stage, err, t_in, t_out);
-        k_batch_step4<POL_TM, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcs, maps, p, buf_out, slot,
-                                                             stage, err, t_in, t_out);
+    if (plain) {
+        if (pol == POL_TE)
+            k_batch_step4<POL_TE, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
+                                                                  stage, err, t_in, t_out);
+        else
+            k_batch_step4<POL_TM, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
+                                                                  stage, err, t_in, t_out);
     }
-    if (n_slots > 0)
-        k_batch_flush4<<<(n_slots + 255) / 256, 256, 0, s>>>(stage, acc, slot_inst, insts, n_slots, t_in);
+    if (accumulate) {
+        if (pol == POL_TE)
+            k_batch_step4<POL_TE, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
+                                                                 stage, err, t_in, t_out);
+        else
+            k_batch_step4<POL_TM, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
+                                                                 stage, err, t_in, t_out);
+        if (n_slots > 0)
+            k_batch_flush4<<<(n_slots + 255) / 256, 256, 0, s>>>(stage, acc, slot_inst, insts, n_slots, t_in);
+    }
     return cudaGetLastError();
 }
 
