@@ -396,12 +396,8 @@ __global__ void __launch_bounds__(NTH, 3)
 // successive changes are <= tol * W and at least min_periods - 1 periods have run, the
 // instance runs one more period, with Fourier accumulation, and stops.  si: the four-step kernel's
 // records, which hold the run lengths too (NULL without them).
-__global__ void k_batch_converge(InstDesc *desc, StreamInst *si, double *energy, double *prev, int *settled,
-                                 const long long *__restrict__ t_next, double tol, int min_periods, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const long long t = *t_next - 1;
-    InstDesc &d = desc[i];
+__device__ void converge(InstDesc &d, StreamInst *si, double *energy, double *prev, int *settled, long long t, double tol,
+                         int min_periods, int i) {
     if (t <= 0 || t >= d.acc_from || (t % (long long)d.period) != 0) return;
     const double W = energy[i];
     energy[i] = 0.0;
@@ -418,6 +414,76 @@ __global__ void k_batch_converge(InstDesc *desc, StreamInst *si, double *energy,
             si[i].steps = d.steps;
         }
     }
+}
+
+// The height of equal row segments of at most `seg` rows: the fewest segments, and none much shorter than
+// the others (200 rows by 64: 4 x 50, not 3 x 64 + 8), so that no unit lasts longer than it must.
+__host__ __device__ inline int even_rows(int ny, int seg) {
+    const int segs = (ny + seg - 1) / seg;
+    return (ny + segs - 1) / segs;
+}
+// The work units of a lattice in such segments.
+__host__ __device__ inline int count_units(int nx, int ny, int seg) {
+    const int rows = even_rows(ny, seg);
+    return ((nx + kStreamOutW - 1) / kStreamOutW) * ((ny + rows - 1) / rows);
+}
+
+// How the four-step kernel's work units are cut: in row segments of at most seg[k] rows, the largest k
+// (shortest segments) whose units still fit the warps that run at once, else seg[0], the
+// height the autotuner chose for the full batch.  A unit lasts as long as its rows and 8 halo
+// rows (about 1 us each), however idle the GPU is, so short segments are the faster ones once
+// the instances that still run leave warps idle; with every warp busy the long ones are, whose
+// halo rows cost less.  16 rows at least: shorter ones spend most of their time on the halo.
+// seg[0] = 0: no four-step launches.
+constexpr int kUnitLevels = 5;
+struct UnitPlan {
+    int seg[kUnitLevels], warps;
+    int4 *units;  // instance, strip, rows from .. to - 1
+    int *n_units;
+};
+
+// One block: the work units of the instances whose run goes past time t (an instance's units in a
+// row, by segment, then strip: neighbouring strips run side by side and share their halo columns
+// in L2).
+__device__ void build_units(const InstDesc *desc, int n, long long t, const UnitPlan &u) {
+    __shared__ int active[kUnitLevels], level, count;
+    if (threadIdx.x < kUnitLevels) active[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (t < desc[i].steps)
+            for (int k = 0; k < kUnitLevels; ++k) atomicAdd(&active[k], count_units(desc[i].nx, desc[i].ny, u.seg[k]));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int k = kUnitLevels - 1;
+        while (k > 0 && (active[k] > u.warps || u.seg[k] >= u.seg[0])) --k;
+        level = k;
+        *u.n_units = active[k];
+        count = 0;
+    }
+    __syncthreads();
+    const int seg = u.seg[level];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        if (t >= desc[i].steps) continue;
+        const int nx = desc[i].nx, ny = desc[i].ny, rows = even_rows(ny, seg);
+        const int strips = (nx + kStreamOutW - 1) / kStreamOutW;
+        int4 *out = u.units + atomicAdd(&count, count_units(nx, ny, seg));
+        for (int y = 0; y < ny; y += rows)
+            for (int st = 0; st < strips; ++st) *out++ = make_int4(i, st, y, min(y + rows, ny));
+    }
+}
+__global__ void __launch_bounds__(1024) k_batch_units(const InstDesc *desc, int n, long long t, const UnitPlan u) {
+    build_units(desc, n, t, u);
+}
+
+// One block: the exits of the step before *t_next, then the units of the instances that still run.
+__global__ void __launch_bounds__(1024) k_batch_converge(InstDesc *desc, StreamInst *si, double *energy, double *prev,
+                                                         int *settled, const long long *__restrict__ t_next, double tol,
+                                                         int min_periods, int n, const UnitPlan u) {
+    const long long t = *t_next - 1;
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        converge(desc[i], si, energy, prev, settled, t, tol, min_periods, i);
+    __syncthreads();
+    if (u.seg[0] > 0) build_units(desc, n, t + 1, u);
 }
 
 // Per-instance stress-tensor integral: block i reduces instance i's contour.
@@ -512,6 +578,7 @@ struct lbm_em_batch {
     // (instance, strip, row segment of at most four_seg rows), per-instance records, tensor maps and
     // source parameters, and the source values of the current launch
     bool four = false;
+    UnitPlan units{};
     int four_seg = 0, four_grid = 0, four_blocks = 0, four_ctas = 0, n_units = 0;
     int4 *d_units = nullptr;
     StreamInst *d_sinsts = nullptr;
@@ -521,8 +588,8 @@ struct lbm_em_batch {
     float *d_stage4 = nullptr;  // staged stencil fields of the accumulating launches (12 per slot)
     int *d_slot_inst = nullptr; // each accumulator slot's instance
     int want_spl = 0;  // lbm_em_batch_opts.steps_per_launch
-    cudaGraphExec_t graph[2][3] = {};  // two launches that start with the state in buf[p], by StepKind
-    long long first_acc = 0, last_plain = 0;  // see batch_kind
+    cudaGraphExec_t graph[2][2] = {};  // two launches that start with the state in buf[p], without and with Fourier sums
+    long long first_acc = 0;           // see batch_accumulates
     bool ran = false;
     // a bounded wait for a tile copy gave up (seen by lbm_em_batch_results): a copy may
     // still have been in flight when its CTA left, so the batch refuses further runs
@@ -614,57 +681,50 @@ static lbm_em_status batch_tiles(lbm_em_batch *b, int tw, int th) {
     return st;
 }
 
-// The height of equal row segments of at most `seg` rows: the fewest segments, and none much shorter than
-// the others (200 rows by 64: 4 x 50, not 3 x 64 + 8), so that no unit lasts longer than it must.
-static int even_rows(int ny, int seg) {
-    const int segs = (ny + seg - 1) / seg;
-    return (ny + segs - 1) / segs;
+// The work units of the instances that still run at time t, on the device.
+static lbm_em_status batch_list_units(lbm_em_batch *b, long long t) {
+    k_batch_units<<<1, std::min(1024, (b->n + 31) / 32 * 32), 0, b->stream>>>(b->d_desc, b->n, t, b->units);
+    return cuda_status(cudaGetLastError(), "listing work units");
 }
 
-// The four-step kernel's work units for row segments of at most `seg` rows: instance by decreasing run
-// length, then segment, then strip (neighbouring strips run side by side and share their halo
-// columns in L2); and the per-instance records with that segment height.
+// The four-step kernel's records, and its work units in segments of at most `seg` rows (UnitPlan).
 static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
-    std::vector<int4> units;
     std::vector<StreamInst> &si = b->sinsts;
     si.resize(b->n);
     for (int i = 0; i < b->n; ++i) {
         const InstDesc &d = b->desc[i];
         StreamInst &r = si[i];
         std::memset(&r, 0, sizeof(r));
-        r.nx = d.nx, r.ny = d.ny, r.pitch = d.pitch, r.kind = d.src.kind;
-        r.seg_rows = even_rows(d.ny, seg), r.n_strips = (d.nx + kStreamOutW - 1) / kStreamOutW, r.ay0 = d.y0, r.ay1 = d.y1;
+        r.nx = d.nx, r.ny = d.ny, r.pitch = d.pitch, r.kind = d.src.kind, r.ay0 = d.y0, r.ay1 = d.y1;
         r.steps = d.steps, r.acc_from = d.acc_from, r.base = (long long)d.base, r.pstride = (long long)d.pstride;
         r.slot_base = (long long)d.slot_base, r.acc_base = d.acc_base, r.period = d.period;
         r.cs = d.src.cs;
         r.runaway = runaway_bits<float>(b->specs[i].E0);
         for (int q = 0; q < 3; ++q) r.m[q] = d.mtabf[q];
     }
-    for (long long ii : b->order) {
-        const int i = (int)ii;
-        for (int y = 0; y < b->desc[i].ny; y += si[i].seg_rows)
-            for (int st = 0; st < si[i].n_strips; ++st) units.push_back(make_int4(i, st, y / si[i].seg_rows, 0));
-    }
+    UnitPlan &u = b->units;
+    u = UnitPlan{{seg, 48, 32, 24, 16}, b->four_grid * kStreamWarps, nullptr, nullptr};
+    b->n_units = 0;
+    for (const InstDesc &d : b->desc) b->n_units += count_units(d.nx, d.ny, seg);
+    const int room = std::max(b->n_units, u.warps);
     dfree(b->d_units);
     b->d_units = nullptr;
-    lbm_em_status st = cuda_status(dmalloc(&b->d_units, units.size() * sizeof(int4)), "cudaMalloc(units)");
-    if (!st)
-        st = cuda_status(copy_async(b->d_units, units.data(), units.size() * sizeof(int4), cudaMemcpyHostToDevice,
-                                    b->stream),
-                         "uploading units");
+    lbm_em_status st = cuda_status(dmalloc(&b->d_units, (size_t)room * sizeof(int4) + sizeof(int)), "cudaMalloc(units)");
+    u.units = b->d_units;
+    u.n_units = (int *)(b->d_units + room);
     if (!st && !b->d_sinsts)
         st = cuda_status(dmalloc(&b->d_sinsts, si.size() * sizeof(StreamInst)), "cudaMalloc(stream records)");
     if (!st)
         st = cuda_status(copy_async(b->d_sinsts, si.data(), si.size() * sizeof(StreamInst), cudaMemcpyHostToDevice,
                                     b->stream),
                          "uploading stream records");
+    if (!st) st = batch_list_units(b, 0);
     if (!st) st = cuda_status(cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");  // pageable sources
-    b->n_units = (int)units.size();
     b->four_seg = seg;
     // one warp per unit: the hardware starts each thread block as an earlier one finishes, which
     // balanced the units better than resident warps walking them (256-instance design map on
     // GB300: 116.7 against 105.4 cells/s, same bits)
-    b->four_blocks = b->four_ctas > 0 ? b->four_ctas * b->sms : (b->n_units + kStreamWarps - 1) / kStreamWarps;
+    b->four_blocks = b->four_ctas > 0 ? b->four_ctas * b->sms : (room + kStreamWarps - 1) / kStreamWarps;
     return st;
 }
 
@@ -703,12 +763,9 @@ static void launch_batch_step2(const lbm_em_batch *b, const BatchArgs<float> &a,
                                                                          b->d_time + p, b->d_time + (1 - p));
 }
 
-// Which instances a four-step launch can find (batch_kind).
-enum StepKind { kPlainOnly, kBoth, kAccOnly };
-
 // One launch from the state in buf[p] (time word p) to buf[1 - p]: one step, two with b->two,
-// four with b->four (kind: of the instances it finds).  The caller alternates p launch by launch.
-static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, StepKind kind = kBoth) {
+// four with b->four (accumulate: see batch_accumulates).  The caller alternates p launch by launch.
+static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, bool accumulate = true) {
     const int grid = b->ctas * b->sms;
     if (b->prec == LBM_EM_F32X2) {
         BatchArgs<df> a{b->d_desc, b->d_tiles, b->n_tiles, b->tile_w, b->tile_h, ilog2(b->tile_w),
@@ -731,10 +788,10 @@ static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, StepKind
                            (const float *)b->buf[p], (float *)b->buf[1 - p], b->d_mat, b->d_slot,
                            b->d_acc, b->d_err, b->d_energy, b->conv_tol > 0.0};
         if (b->four) {
-            launch_batch_step4(b->d_sinsts, b->d_srcp, b->d_units, b->n_units, b->d_smaps4, p,
+            launch_batch_step4(b->d_sinsts, b->d_srcp, b->units.units, b->units.n_units, b->d_smaps4, p,
                                (float *)b->buf[1 - p], b->d_slot, b->d_acc, b->d_stage4, b->d_slot_inst,
                                (int)b->acc_slots, b->d_err, b->d_time + p, b->d_time + (1 - p), b->four_blocks,
-                               b->pol, kind != kAccOnly, kind != kPlainOnly, s);
+                               b->pol, accumulate, s);
         } else if (b->two) {
             k_batch_source<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->n, b->d_time + p, b->d_srcs);
             if (b->pol == POL_TE)
@@ -749,8 +806,9 @@ static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, StepKind
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && b->conv_tol > 0.0 && !b->four) {  // (no period boundary inside a four-step launch)
-        k_batch_converge<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->d_sinsts, b->d_energy, b->d_prev, b->d_settled,
-                                                           b->d_time + (1 - p), b->conv_tol, b->min_periods, b->n);
+        k_batch_converge<<<1, std::min(1024, (b->n + 31) / 32 * 32), 0, s>>>(
+            b->d_desc, b->d_sinsts, b->d_energy, b->d_prev, b->d_settled, b->d_time + (1 - p), b->conv_tol,
+            b->min_periods, b->n, b->units);
         e = cudaGetLastError();
     }
     return e;
@@ -798,28 +856,25 @@ static bool conv_four(const lbm_em_batch *b) {
     return 2 * in4 >= b->max_steps;
 }
 
-// The instances that `n` four-step launches from time t can find.  first_acc: the earliest time that an
-// accumulated period can begin at; last_plain: the latest.  With convergence exits that is
-// decided on the device, but never before the third sample (k_batch_converge compares two
-// changes) or min_periods, and never after the nominal time.
-static StepKind batch_kind(const lbm_em_batch *b, long long t, int n) {
-    if (t + 4 * n - 1 < b->first_acc) return kPlainOnly;
-    return t + 3 >= b->last_plain ? kAccOnly : kBoth;
-}
+// Whether `n` four-step launches from time t may find an instance in its accumulated period.
+// first_acc: the earliest time that one can begin at.  With convergence exits that is decided on the
+// device, but never before the third sample (k_batch_converge compares two changes) or
+// min_periods.
+static bool batch_accumulates(const lbm_em_batch *b, long long t, int n) { return t + 4 * n - 1 >= b->first_acc; }
 
 // The graph of two launches that starts with the state in buf[p].
-static lbm_em_status batch_capture(lbm_em_batch *b, int p, StepKind kind) {
+static lbm_em_status batch_capture(lbm_em_batch *b, int p, bool accumulate) {
     cudaGraph_t g = nullptr;
     lbm_em_status st = cuda_status(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
     if (st) return st;
-    cudaError_t e = batch_launch(b, b->cap, p, kind);
-    if (e == cudaSuccess) e = batch_launch(b, b->cap, 1 - p, kind);
+    cudaError_t e = batch_launch(b, b->cap, p, accumulate);
+    if (e == cudaSuccess) e = batch_launch(b, b->cap, 1 - p, accumulate);
     cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return cuda_status(e != cudaSuccess ? e : e2, "capturing the batch graph");
     }
-    e = cudaGraphInstantiate(&b->graph[p][kind], g, 0);
+    e = cudaGraphInstantiate(&b->graph[p][accumulate], g, 0);
     cudaGraphDestroy(g);
     return cuda_status(e, "cudaGraphInstantiate");
 }
@@ -1081,7 +1136,6 @@ lbm_em_status lbm_em_batch_create(const lbm_em_instance *specs, int32_t n, const
     for (const InstDesc &d : b->desc) {
         const long long exit = o->conv_tol > 0.0 ? (long long)std::max(3, o->min_periods - 1) * d.period + 1 : LLONG_MAX;
         b->first_acc = std::min(b->first_acc, std::min(d.acc_from, exit));
-        b->last_plain = std::max(b->last_plain, d.acc_from);
     }
     b->buf_elems = base;
     b->mat_bytes = mat;
@@ -1244,20 +1298,29 @@ lbm_em_status lbm_em_batch_run(lbm_em_batch_t *b) {
     const long long spl = batch_spl(b), per_graph = 2 * spl;
     const bool stops = b->four && b->conv_tol > 0.0;
     long long t = 0;
-    int p = 0;
+    int p = 0, running = b->n;  // of b->order (by decreasing run length), how many still run at the last listing
+    if (b->four) {
+        st = batch_list_units(b, 0);
+        if (st) return st;
+    }
     while (t < b->max_steps) {
         long long left = stops ? conv_gap(b, t) : b->max_steps - t;
         for (; left >= per_graph; left -= per_graph, t += per_graph) {
-            const StepKind kind = b->four ? batch_kind(b, t, 2) : kBoth;
-            if (!b->graph[p][kind]) {
-                st = batch_capture(b, p, kind);
+            const bool accumulate = !b->four || batch_accumulates(b, t, 2);
+            if (b->four && !stops && b->desc[(int)b->order[running - 1]].steps <= t) {  // shorter runs have ended
+                while (b->desc[(int)b->order[running - 1]].steps <= t) --running;
+                st = batch_list_units(b, t);
                 if (st) return st;
             }
-            st = cuda_status(cudaGraphLaunch(b->graph[p][kind], b->stream), "cudaGraphLaunch");
+            if (!b->graph[p][accumulate]) {
+                st = batch_capture(b, p, accumulate);
+                if (st) return st;
+            }
+            st = cuda_status(cudaGraphLaunch(b->graph[p][accumulate], b->stream), "cudaGraphLaunch");
             if (st) return st;
         }
         if (spl > 1 && left >= spl) {
-            st = cuda_status(batch_launch(b, b->stream, p, b->four ? batch_kind(b, t, 1) : kBoth), "batch step");
+            st = cuda_status(batch_launch(b, b->stream, p, !b->four || batch_accumulates(b, t, 1)), "batch step");
             if (st) return st;
             p ^= 1;
             left -= spl;

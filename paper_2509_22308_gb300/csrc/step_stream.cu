@@ -681,20 +681,20 @@ __global__ void __launch_bounds__(NW * 32, 3)
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.err, kErrUnstable);
 }
 
-// Batched design maps: the warps walk the work units of every instance (instance, strip, row
-// segment; ordered by decreasing run length, then segment, then strip) with a grid stride,
-// skipping instances that have finished, four steps per launch; the batch launches one warp per
-// unit, so each warp normally takes one.  Two instantiations split the unfinished instances between
-// them, one after the other where a launch can have both kinds (launch_batch_step4): ACC = false takes those with
-// no time of their accumulated (last) period among the launch's four, ACC = true the others,
-// whose stencil sites' fields it stages for the levels whose time falls in that period
-// (k_batch_flush4 adds them to the Fourier sums after it; ACC = true takes the general row
-// loop).  An instance that ends inside a launch runs on past its end without accumulating; its
-// state is not needed afterwards.  FP32.
+// Batched design maps: the warps walk the work units of the unfinished instances with a grid
+// stride, four steps per launch; the batch launches at least a warp per unit, so each normally
+// takes one.  ACC: some instances may have
+// times of their accumulated (last) period among the launch's four; their units take the general row
+// loop and stage the stencil sites' fields for those times (k_batch_flush4 adds them to the Fourier
+// sums after the launch), the other instances' units run beside them as without ACC.  (As a
+// launch of their own after the others, the few accumulating instances of a map with
+// convergence exits doubled a launch's time: one unit lasts as long as a full GPU of them.)  An
+// instance that ends inside a launch runs on past its end without accumulating; its state is not
+// needed afterwards.  FP32.
 template <int POL, bool ACC>
 __global__ void __launch_bounds__(NW * 32, 3)
-    k_batch_step4(const StreamInst *__restrict__ insts, const int4 *__restrict__ units, int n_units,
-                  const SourceParams *__restrict__ srcp, const CUtensorMap *__restrict__ maps, int p,
+    k_batch_step4(const StreamInst *__restrict__ insts, const int4 *__restrict__ units,
+                  const int *__restrict__ n_units, const SourceParams *__restrict__ srcp, const CUtensorMap *__restrict__ maps, int p,
                   float *__restrict__ buf_out, const int *__restrict__ slot, float *__restrict__ stage,
                   unsigned *__restrict__ err, const long long *__restrict__ t_in, long long *__restrict__ t_out) {
     using LY = Layout<false>;
@@ -716,12 +716,13 @@ __global__ void __launch_bounds__(NW * 32, 3)
     }
     __syncthreads();  // the only block-wide barrier
     RingState R{ring, bars[warp], reinterpret_cast<float4 *>(ring + RING * LY::SLOT), 0, 0u};
-    const int stride = (int)gridDim.x * NW;
-    for (int w = (int)blockIdx.x * NW + warp; w < n_units; w += stride) {
+    const int stride = (int)gridDim.x * NW, end = *n_units;
+    for (int w = (int)blockIdx.x * NW + warp; w < end; w += stride) {
         const int4 un = units[w];
         const StreamInst &I = insts[un.x];
         const long long steps = I.steps;
-        if (t >= steps || (t + BT - 1 >= I.acc_from) != ACC) continue;  // uniform over the warp
+        if (t >= steps) continue;  // uniform over the warp, like acc
+        const bool acc = ACC && t + BT - 1 >= I.acc_from;
         __syncwarp();              // the previous unit's reads of the table and context are done
         if (lane < 3) wtab[warp][lane] = I.m[lane];
         UnitCtx &u = uctx[warp];
@@ -745,8 +746,8 @@ __global__ void __launch_bounds__(NW * 32, 3)
         UnitRun &r = urun[warp];
         if (lane == 0) {
             r.xs = un.y * OUTW - HALO;
-            r.y0 = un.z * I.seg_rows;
-            r.y1 = min(r.y0 + I.seg_rows, I.ny);
+            r.y0 = un.z;
+            r.y1 = un.w;
             r.t = t;
             r.smap = maps + 3 * un.x + p;
             r.fmap = r.smap;
@@ -760,7 +761,11 @@ __global__ void __launch_bounds__(NW * 32, 3)
         if (un.y == 0 && I.kind != SRC_NONE) source_levels_f(srcp[un.x], t, &sp[warp]);
         __syncwarp();
         bool bad = false;
-        const bool ok = stream_unit<false, POL, ACC, !ACC>(u, r, R, bad);
+        bool ok;
+        if (ACC && acc)
+            ok = stream_unit<false, POL, true, false>(u, r, R, bad);
+        else
+            ok = stream_unit<false, POL, false, true>(u, r, R, bad);
         if (!ok) {  // a row copy never completed: report, leave
             if (lane == 0) atomicOr(err + un.x, kErrTimeout);
             return;
@@ -950,30 +955,20 @@ cudaError_t encode_batch_stream_maps(CUtensorMap *maps, const float *buf0, const
     return e;
 }
 
-cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, const int4 *units, int n_units,
-                               const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
+cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, const int4 *units,
+                               const int *n_units, const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
                                float *stage, const int *slot_inst, int n_slots, unsigned *err, const long long *t_in,
-                               long long *t_out, int grid, int pol, bool plain, bool accumulate, cudaStream_t s) {
+                               long long *t_out, int grid, int pol, bool accumulate, cudaStream_t s) {
     const size_t sm = Layout<false>::SMEM;
-    // both write t + 4 to t_out; neither reads it
-    if (plain) {
-        if (pol == POL_TE)
-            k_batch_step4<POL_TE, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
-                                                                  stage, err, t_in, t_out);
-        else
-            k_batch_step4<POL_TM, false><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
-                                                                  stage, err, t_in, t_out);
-    }
-    if (accumulate) {
-        if (pol == POL_TE)
-            k_batch_step4<POL_TE, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
-                                                                 stage, err, t_in, t_out);
-        else
-            k_batch_step4<POL_TM, true><<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot,
-                                                                 stage, err, t_in, t_out);
-        if (n_slots > 0)
-            k_batch_flush4<<<(n_slots + 255) / 256, 256, 0, s>>>(stage, acc, slot_inst, insts, n_slots, t_in);
-    }
+    auto run = [&](auto kernel) {
+        kernel<<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot, stage, err, t_in, t_out);
+    };
+    if (accumulate)
+        pol == POL_TE ? run(k_batch_step4<POL_TE, true>) : run(k_batch_step4<POL_TM, true>);
+    else
+        pol == POL_TE ? run(k_batch_step4<POL_TE, false>) : run(k_batch_step4<POL_TM, false>);
+    if (accumulate && n_slots > 0)
+        k_batch_flush4<<<(n_slots + 255) / 256, 256, 0, s>>>(stage, acc, slot_inst, insts, n_slots, t_in);
     return cudaGetLastError();
 }
 

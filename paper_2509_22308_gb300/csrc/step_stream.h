@@ -45,14 +45,14 @@ struct SrcLevels {
 // table (vacuum, region II, region III) in FP32.
 struct alignas(16) StreamInst {
     int nx, ny, pitch, kind;
-    int seg_rows, n_strips, ay0, ay1;
+    int ay0, ay1;
     long long steps, acc_from;
     long long base, pstride;
     long long slot_base;
     int acc_base, period;
     const double2 *cs;
     unsigned runaway;
-    int pad;
+    int pad[3];
     MatT<float> m[3];
 };
 
@@ -61,18 +61,16 @@ cudaError_t batch_stream_prepare(int *resident_warps);
 // The three tensor maps of one instance (state in buffer 0, in buffer 1, ids) in maps[0..2].
 cudaError_t encode_batch_stream_maps(CUtensorMap *maps, const float *buf0, const float *buf1, const uint8_t *ids,
                                      int nx, int ny, int pitch, size_t pstride);
-// Four steps of every unfinished instance: the kernel over units[n_units] (int4: instance, strip,
-// segment; walked with a stride of grid x kStreamWarps warps), source parameters srcp[i] of
-// instance i, input state buffer p (maps[3 i + p]), output buf_out; the stencil sites of instances
-// in their accumulated period staged in stage (12 floats per slot of the packed accumulators
-// acc[6 n_slots]) and added to acc by a flush over the slots (slot_inst[n_slots]: each slot's
-// instance).  plain: some instance may be before its accumulated period at all four times;
-// accumulate: some may be in it.  At least one holds, and a kernel that would find no
-// instance is not launched.
-cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, const int4 *units, int n_units,
-                               const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
+// Four steps of every unfinished instance: the kernel over units[*n_units] (int4: instance,
+// strip, rows from .. to - 1; walked with a stride of grid x kStreamWarps warps), source parameters srcp[i] of instance i, input state buffer p
+// (maps[3 i + p]), output buf_out.  accumulate: some instances may be in their accumulated period
+// at one of the four times; their stencil sites are staged in stage (12 floats per slot of the
+// packed accumulators acc[6 n_slots]) and added to acc by a flush over the slots
+// (slot_inst[n_slots]: each slot's instance).
+cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp, const int4 *units,
+                               const int *n_units, const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
                                float *stage, const int *slot_inst, int n_slots, unsigned *err, const long long *t_in,
-                               long long *t_out, int grid, int pol, bool plain, bool accumulate, cudaStream_t s);
+                               long long *t_out, int grid, int pol, bool accumulate, cudaStream_t s);
 
 // Four steps: the state described by the maps (time word t_in) -> fout / the FP16-deviation
 // output planes of fa (t_out = t + 4).  FP32 of either polarization (a.pol), or the

@@ -55,3 +55,19 @@ def test_many_different_periods_keep_one_step_launches():
         assert np.array_equal(b.steps(), c.steps()) and np.array_equal(b.results()[0], c.results()[0])
     finally:
         b.close(), c.close()
+
+
+@pytest.mark.parametrize("n", [1, 33, 60])
+def test_shorter_segments_as_runs_end(n):
+    """Units of 16 rows from the start (one instance), and longer ones that shorten as runs of 2 to 10
+    periods end: forces equal the one-step kernel's bits."""
+    insts = [_inst(150 + 7 * (k % 9), 260 - 11 * (k % 7), 20 + k % 3, 2 + k % 9) for k in range(n)]
+    F = []
+    for spl in (4, 1):
+        b = L.Batch(insts, "f32", steps_per_launch=spl)
+        try:
+            b.run()
+            F.append(b.results()[0])
+        finally:
+            b.close()
+    assert np.array_equal(F[0], F[1])
