@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "pair32.cuh"
+#include "pairdf.cuh"
 #include "resident.h"
 #include "tma.cuh"
 
@@ -827,13 +828,15 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         return true;
     };
 
-    // All steps of the warp, rows downwards or upwards.  Returns false after a wait gave up.
+    // All steps of the warp, rows downwards or upwards.  Returns false after a wait gave up.  dir is a
+    // constant in FP64, where it is compiled twice, and a value in double-float, whose two copies of the
+    // long update would not fit the instruction cache.
     auto steps = [&](auto dir) -> bool {
-        constexpr bool DOWN = decltype(dir)::value;
+        const bool DOWN = dir;
         // planes that come from the row taken before (carried) and from the row taken next
-        constexpr int PC0 = DOWN ? P_EPY : P_EMY, PC1 = DOWN ? P_HYPY : P_HYMY;
-        constexpr int PN0 = DOWN ? P_EMY : P_EPY, PN1 = DOWN ? P_HYMY : P_HYPY;
-        constexpr int RS = (DOWN ? 1 : -1) * NPLANES * 32;
+        const int PC0 = DOWN ? P_EPY : P_EMY, PC1 = DOWN ? P_HYPY : P_HYMY;
+        const int PN0 = DOWN ? P_EMY : P_EPY, PN1 = DOWN ? P_HYMY : P_HYPY;
+        const int RS = (DOWN ? 1 : -1) * NPLANES * 32;
         const RowLink<V> &la = DOWN ? up : dn, &lb = DOWN ? dn : up;
         const int ifirst = DOWN ? 0 : nrows - 1;
         for (int k = 0; k < r.n; ++k) {
@@ -846,15 +849,17 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
             if (la.exists && !receive(la, k, c0, c1)) return false;
             V *const eout = edge + (k & 1) * bstep + loc * 128 + lane;
             Msg *const xs = x_send + (so & 1u) * xslot;
-            for (int j = 0, i = ifirst; j < nrows; ++j, i += DOWN ? 1 : -1, q += RS) {
-                const bool lastrow = j + 1 == nrows;
-                V n0, n1;
-                if (!lastrow) {
-                    n0 = q[RS + PN0 * 32], n1 = q[RS + PN1 * 32];
-                } else {
-                    n0 = q[PN0 * 32], n1 = q[PN1 * 32];
-                    if (lb.exists && !receive(lb, k, n0, n1)) return false;
+            // the pair that row i (at w) pulls from the row taken after it; false: gave up
+            auto next = [&](const V *w, bool last, V &n0, V &n1) -> bool {
+                if (!last) {
+                    n0 = w[RS + PN0 * 32], n1 = w[RS + PN1 * 32];
+                    return true;
                 }
+                n0 = w[PN0 * 32], n1 = w[PN1 * 32];
+                return !lb.exists || receive(lb, k, n0, n1);
+            };
+            // row i (at w) pulled from its neighbours, and its own pair carried to the row taken after it
+            auto pull = [&](const V *w, int i, V n0, V n1, Pop<V> &p) -> bool {
                 // the border values from the left (lane 0) and the right (lane 31)
                 T in0{}, in1{};
                 if (inner) {
@@ -863,17 +868,16 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                     while (!__all_sync(kFull, !waits_x || get_site<T>(xr, in0, in1, seq)))
                         if (pt.over(a.err)) return false;
                 }
-                Pop<V> p;
-                const V epx = q[P_EPX * 32], emx = q[P_EMX * 32], hxpx = q[P_HXPX * 32], hxmx = q[P_HXMX * 32];
-                p.ez = q[P_EZ * 32];
-                p.hxz = q[P_HXZ * 32];
-                p.hyz = q[P_HYZ * 32];
+                const V epx = w[P_EPX * 32], emx = w[P_EMX * 32], hxpx = w[P_HXPX * 32], hxmx = w[P_HXMX * 32];
+                p.ez = w[P_EZ * 32];
+                p.hxz = w[P_HXZ * 32];
+                p.hyz = w[P_HYZ * 32];
                 p.epy = DOWN ? c0 : n0;
                 p.hypy = DOWN ? c1 : n1;
                 p.emy = DOWN ? n0 : c0;
                 p.hymy = DOWN ? n1 : c1;
-                c0 = q[PC0 * 32];
-                c1 = q[PC1 * 32];
+                c0 = w[PC0 * 32];
+                c1 = w[PC1 * 32];
                 if (strip == 0 && lane == 0) in0 = epx, in1 = hxpx;
                 p.epx = from_left(epx, in0, lane);
                 p.hxpx = from_left(hxpx, in1, lane);
@@ -883,11 +887,11 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                     p.emx = keep_last(p.emx, emx, a_last, b_last);
                     p.hxmx = keep_last(p.hxmx, hxmx, a_last, b_last);
                 }
-                if (src_now && lane == 0) {
-                    inject_source_t<T>(kind, srcv[2 * k], srcv[2 * k + 1], p);
-                }
-                T f3[3];
-                update_row<POL, ACC>(p, uniform ? mu : table[ids[i * 32 + lane]], a.runaway, in_a, rw, f3);
+                if (src_now && lane == 0) inject_source_t<T>(kind, srcv[2 * k], srcv[2 * k + 1], p);
+                return true;
+            };
+            // the updated row i (to w): its fields staged, its populations kept and sent
+            auto put = [&](V *w, int i, const Pop<V> &p, const T *f3) {
                 if constexpr (ACC) {
                     const int y = y0 + i;
                     if (y >= a.accp.y0 && y <= a.accp.y1) {
@@ -899,44 +903,79 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                         }
                     }
                 }
-                q[P_EZ * 32] = p.ez;
-                q[P_EPX * 32] = p.epx;
-                q[P_EMX * 32] = p.emx;
-                q[P_EPY * 32] = p.epy;
-                q[P_EMY * 32] = p.emy;
-                q[P_HXPX * 32] = p.hxpx;
-                q[P_HXMX * 32] = p.hxmx;
-                q[P_HXZ * 32] = p.hxz;
-                q[P_HYPY * 32] = p.hypy;
-                q[P_HYMY * 32] = p.hymy;
-                q[P_HYZ * 32] = p.hyz;
-                if (sends) {
-                    if (sends_x)
-                        send_site(xs + (size_t)i * 2, lane == 0 ? p.emx : p.epx, lane == 0 ? p.hxmx : p.hxpx, so);
-                    if (i == 0 && has_up) {
-                        if (up_here) {
-                            eout[0] = p.emy, eout[32] = p.hymy;
-                            __syncwarp();
-                            if (lane == 0) flag_set(flags + 2 * loc, (unsigned)k + 1u);
-                        } else {
-                            send_row(up_send + (so & 1u) * yslot, p.emy, p.hymy, so);
-                        }
+                w[P_EZ * 32] = p.ez;
+                w[P_EPX * 32] = p.epx;
+                w[P_EMX * 32] = p.emx;
+                w[P_EPY * 32] = p.epy;
+                w[P_EMY * 32] = p.emy;
+                w[P_HXPX * 32] = p.hxpx;
+                w[P_HXMX * 32] = p.hxmx;
+                w[P_HXZ * 32] = p.hxz;
+                w[P_HYPY * 32] = p.hypy;
+                w[P_HYMY * 32] = p.hymy;
+                w[P_HYZ * 32] = p.hyz;
+                if (!sends) return;
+                if (sends_x)
+                    send_site(xs + (size_t)i * 2, lane == 0 ? p.emx : p.epx, lane == 0 ? p.hxmx : p.hxpx, so);
+                if (i == 0 && has_up) {
+                    if (up_here) {
+                        eout[0] = p.emy, eout[32] = p.hymy;
+                        __syncwarp();
+                        if (lane == 0) flag_set(flags + 2 * loc, (unsigned)k + 1u);
+                    } else {
+                        send_row(up_send + (so & 1u) * yslot, p.emy, p.hymy, so);
                     }
-                    if (i == nrows - 1 && has_down) {
-                        if (down_here) {
-                            eout[64] = p.epy, eout[96] = p.hypy;
-                            __syncwarp();
-                            if (lane == 0) flag_set(flags + 2 * loc + 1, (unsigned)k + 1u);
-                        } else {
-                            send_row(down_send + (so & 1u) * yslot, p.epy, p.hypy, so);
-                        }
+                }
+                if (i == nrows - 1 && has_down) {
+                    if (down_here) {
+                        eout[64] = p.epy, eout[96] = p.hypy;
+                        __syncwarp();
+                        if (lane == 0) flag_set(flags + 2 * loc + 1, (unsigned)k + 1u);
+                    } else {
+                        send_row(down_send + (so & 1u) * yslot, p.epy, p.hypy, so);
                     }
+                }
+            };
+            for (int j = 0, i = ifirst; j < nrows; ++j, i += DOWN ? 1 : -1, q += RS) {
+                V n0, n1;
+                Pop<V> p;
+                T f3[3];
+                if constexpr (std::is_same<T, df>::value) {
+                    // two rows at a time as packed pairs (an odd last one with itself).  The first is sent no
+                    // earlier than the second has what it needs of the step before, which waits for
+                    // nothing of this step.
+                    const bool pair = j + 1 < nrows;
+                    const int i2 = pair ? i + (DOWN ? 1 : -1) : i;
+                    if (!next(q, !pair, n0, n1) || !pull(q, i, n0, n1, p)) return false;
+                    Pop<V> p2 = p;
+                    if (pair && (!next(q + RS, j + 2 == nrows, n0, n1) || !pull(q + RS, i2, n0, n1, p2))) return false;
+                    Pop<df2> v;
+                    df2 g3[3];
+                    each_of_pair(v, p, p2, [](df2 &o, df &u, df &w) { o = pack_df(u, w); });
+                    rw |= update_pair<POL, ACC>(v, uniform ? mu : table[ids[i * 32 + lane]],
+                                                uniform ? mu : table[ids[i2 * 32 + lane]], true, a.runaway, g3) &&
+                          in_a;
+                    each_of_pair(v, p, p2, [](df2 &o, df &u, df &w) { u = first(o), w = second(o); });
+                    if (ACC) f3[0] = first(g3[0]), f3[1] = first(g3[1]), f3[2] = first(g3[2]);
+                    put(q, i, p, f3);
+                    if (!pair) break;
+                    if (ACC) f3[0] = second(g3[0]), f3[1] = second(g3[1]), f3[2] = second(g3[2]);
+                    put(q + RS, i2, p2, f3);
+                    ++j, i = i2, q += RS;
+                } else {
+                    if (!next(q, j + 1 == nrows, n0, n1) || !pull(q, i, n0, n1, p)) return false;
+                    update_row<POL, ACC>(p, uniform ? mu : table[ids[i * 32 + lane]], a.runaway, in_a, rw, f3);
+                    put(q, i, p, f3);
                 }
             }
         }
         return true;
     };
-    const bool ok = down ? steps(std::true_type{}) : steps(std::false_type{});
+    bool ok;
+    if constexpr (std::is_same<T, df>::value)
+        ok = steps(down);
+    else
+        ok = down ? steps(std::true_type{}) : steps(std::false_type{});
 
     if (!ok) {
         if (lane == 0) atomicOr(a.err, kErrTimeout);
@@ -1061,9 +1100,10 @@ cudaError_t resident_plan(int nx, int ny, ResidentPlan *plan) {
             fits = p.warps + p.comm <= kResidentMaxWarps && p.rows <= kResidentMaxRows && p.smem <= (size_t)smem_max;
             if (fits) break;
         }
-        // double-float (600 FP32 operations per site) is bound by those soon: with more than one row per warp
-        // the one-step kernel is as fast (us per step here / there: 256^2 3.7 / 5.2, 320^2 4.9 / 5.2, 448^2 8.6 / 7.6)
-        if (std::is_same<T, df>::value && p.rows > 1) fits = false;
+        // double-float (576 FP32 operations per site) is bound by their latency at the few warps that the
+        // registers leave, so with more than one pair of rows per warp the one-step kernel is the faster one
+        // (us per step here / there: 256^2 3.7 / 4.7, 320^2 4.0 / 4.8, 384^2 6.3 / 5.6, 512^2 9.0 / 8.0)
+        if (std::is_same<T, df>::value && p.rows > 2) fits = false;
     }
     if (!fits) return cudaSuccess;
     p.ctas = (p.total + p.warps - 1) / p.warps;

@@ -1,8 +1,11 @@
 // Fused stream-collide step of the D3Q7 Maxwell lattice Boltzmann scheme
 // (arXiv 2509.22308, Sec. III) for the FP64 and FP32 storage forms and both
 // polarizations, plus the kernel that reconstructs the fields at the current time.
+#include <type_traits>
+
 #include "common.cuh"
 #include "launchers.h"
+#include "pairdf.cuh"
 
 namespace lbmem {
 
@@ -42,6 +45,42 @@ __global__ void __launch_bounds__(BX *BY) k_step(const StepArgs<T> a, const T *_
     store_site(fout, a.pstride, idx, p);
 }
 
+// The double-float step without Fourier sums: each thread takes the sites of one column in two adjacent
+// rows as packed pairs (pairdf.cuh), which halves the instructions that bound the scalar kernel;
+// from 512^2 on the state's way through L2 and HBM (177 bytes per update) bounds this one.  GLUPS, scalar
+// and this: 512^2 29.9 and 33.0, 768^2 33.8 and 36.5, 1024^2 29.2 and 31.7.  Blocks of two warps at 96
+// registers: blocks of four 1.5 % slower at 512^2, more registers 4 %.
+constexpr int DFY = 2;  // pairs of rows per block
+template <int POL>
+__global__ void __launch_bounds__(BX *DFY, 10) k_step_df(const StepArgs<df> a, const df *__restrict__ fin,
+                                                        df *__restrict__ fout, const long long *__restrict__ t_in,
+                                                        long long *__restrict__ t_out) {
+    const int x = blockIdx.x * BX + threadIdx.x;
+    const int y = 2 * (blockIdx.y * DFY + threadIdx.y);
+    const long long t = *t_in;
+    if (x == 0 && y == 0) *t_out = t + 1;
+    if (x >= a.nx || y >= a.ny) return;
+    const bool two = y + 1 < a.ny;
+    const int yb = two ? y + 1 : y;  // the last row of an odd number is computed twice, stored once
+    Pop<df> pa, pb;
+    pull_planes(a, fin, x, y, pa);
+    pull_planes(a, fin, x, yb, pb);
+    if (x == 0 && t >= 1 && a.src.kind != SRC_NONE) {
+        double g, inc;
+        source_values(a.src, t, &g, &inc);
+        inject_source(a.src.kind, g, inc, pa);
+        inject_source(a.src.kind, g, inc, pb);
+    }
+    const size_t idx = (size_t)y * a.pitch + x, idb = (size_t)yb * a.pitch + x;
+    const MatT<df> ma = a.mtab[a.mat[idx]], mb = a.mtab[a.mat[idb]];
+    Pop<df2> p;
+    each_of_pair(p, pa, pb, [](df2 &v, df &u, df &w) { v = pack_df(u, w); });
+    if (update_pair<POL>(p, ma, mb, two, a.runaway)) atomicOr(a.err, 1u);
+    each_of_pair(p, pa, pb, [](df2 &v, df &u, df &w) { u = first(v), w = second(v); });
+    store_site(fout, a.pstride, idx, pa);
+    if (two) store_site(fout, a.pstride, idb, pb);
+}
+
 // The field triple at time *t_dev (pull + moments, no collision), packed [ny][nx]:
 // TM E_z, H_x, H_y; TE H_z, E_x, E_y.
 template <typename T, int POL>
@@ -65,6 +104,15 @@ __global__ void __launch_bounds__(BX *BY) k_fields(const StepArgs<T> a, const T 
 template <typename T>
 cudaError_t launch_step(const StepArgs<T> &a, const T *fin, T *fout, const long long *t_in,
                         long long *t_out, bool accumulate, cudaStream_t s) {
+    if constexpr (std::is_same<T, df>::value)
+        if (!accumulate) {
+            const dim3 grid((a.nx + BX - 1) / BX, (a.ny + 2 * DFY - 1) / (2 * DFY)), block(BX, DFY);
+            if (a.pol == POL_TE)
+                k_step_df<POL_TE><<<grid, block, 0, s>>>(a, fin, fout, t_in, t_out);
+            else
+                k_step_df<POL_TM><<<grid, block, 0, s>>>(a, fin, fout, t_in, t_out);
+            return cudaGetLastError();
+        }
     dim3 grid((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY), block(BX, BY);
     if (a.pol == POL_TE) {
         if (accumulate)
