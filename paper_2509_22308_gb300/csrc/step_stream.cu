@@ -57,6 +57,7 @@ constexpr unsigned ROW32 = NPLANES * LW * 4;   // FP32 state row: 11 planes x 64
 constexpr int DEVW = LW + 8, DEVOFF = 4;
 constexpr unsigned ROWDEV = NPLANES * DEVW * 2;
 constexpr unsigned ROWFLD = 3 * LW * 4;        // FP32 fields row: 3 planes x 64 floats
+constexpr int PAIR_IDS = 4;  // batches: ids are below it, and pairs of them index a table
 constexpr size_t r128(size_t b) { return (b + 127) / 128 * 128; }
 static_assert(LW == 64 && OUTW + 2 * HALO == LW && HALO % 4 == 0 && HALO >= BT,
               "two sites per lane, a 16-byte aligned halo as wide as the steps");
@@ -277,7 +278,8 @@ struct UnitRun {
     int xs, y0, y1;
     long long t;
     const CUtensorMap *smap, *fmap, *imap;
-    const MatT<float> *table;
+    const MatT<float> *table;  // by id
+    const PairMat *pairs;      // PAIRS: by id of site A + PAIR_IDS x id of site B
     const float *src_g, *src_inc;
 };
 
@@ -303,8 +305,10 @@ __device__ __forceinline__ void stage_owned(float *stage, int sl, int k, float f
 }
 
 // Four steps of one work unit (see the top of this file).  Returns false after a bounded wait
-// for a row copy gave up.  bad: set when a stored site's field ran away.  SPLIT: the
-// steady-state rows take the copies of the row loop without the general loop's tests.  ACC:
+// for a row copy gave up.  bad: set when a stored site's field ran away.  SPLIT: how many copies of the
+// row loop without the general loop's tests the steady-state rows take (see the end).  PAIRS: the
+// table is one of pairs of materials (3 regions in a batch: two loads a row and level less, 105.0 -> 101.5
+// ms on 180 instances of 160^2; a single lattice has up to 256 materials).  ACC:
 // instead of adding each stencil site's Fourier terms to its FP64 sums, store its FP32 fields at
 // level k to stage[12 slot + 3 k ..] (u.stage); a flush kernel adds them after the launch in the
 // same order and arithmetic as one step per launch.  Adding them here cost a few FP64
@@ -317,7 +321,7 @@ __device__ __forceinline__ void stage_owned(float *stage, int sl, int k, float f
 // 239.6 to 242.7, FP16-deviation and batches even.  Keeping a row pair's material constants from
 // level to level (reloaded where a vote finds other ids) spilled and lost: 2048^2 203.0, a batch
 // of 180 instances of 160^2 28 % slower.
-template <bool F16, int POL, bool ACC, bool SPLIT, bool MIX = false>
+template <bool F16, int POL, bool ACC, int SPLIT, bool MIX = false, bool PAIRS = false>
 __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, RingState &R, bool &bad) {
     // the steady-state copies treat every computed row as owned, which holds for the stored level
     // only: the Fourier sums of the levels before it would count halo rows twice
@@ -451,6 +455,7 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
                     else
                         pull_row(c0, ey, hy, my, mh, xa0, xa_last, xb_last, c);
                     idq = *reinterpret_cast<const unsigned short *>(sq + LY::IDS + idoff + 2 * lane);
+                    if (PAIRS) idq = ((idq & 0xffu) + (idq >> 8) * PAIR_IDS) * (unsigned)sizeof(PairMat);
                     id_k0 = idq;
                 } else {
                     f2 ey, hy, my, mh;
@@ -479,7 +484,11 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
                         c.hxpx = pack2(0.f, hi2(c.hxpx));
                     }
                 }
-                const PairMat mat = pair_mat(r.table[idq & 0xffu], r.table[(idq >> 8) & 0xffu]);
+                PairMat mat;
+                if constexpr (PAIRS)  // the pair's byte offset, formed once per row
+                    mat = *reinterpret_cast<const PairMat *>(reinterpret_cast<const char *>(r.pairs) + idq);
+                else
+                    mat = pair_mat(r.table[idq & 0xffu], r.table[(idq >> 8) & 0xffu]);
                 const bool owned = out_lane && (FAST || (q >= y0 && q < y1));
                 const bool store = k == BT - 1 && owned;
                 // ACC: a row of contour stencil sites in the accumulated period (uniform over the warp)
@@ -586,14 +595,17 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
         return true;
     };
 
-    // With SPLIT, the steady-state rows (every level computes and stores, no lattice top or
+    // With SPLIT 2, the steady-state rows (every level computes and stores, no lattice top or
     // bottom, no segment end) run copies of the row without those tests: one for interior strips,
     // without the left and right edge tests too, one for the two strips at the lattice's edges.
     // Measured on GB300 (GLUPS on 8192^2 / 2048^2): FP32 with the general loop for every row
     // 240.1 / 180.3, with both copies 257.2 / 195.0; FP16-deviation with the interior copy only
     // (the edge strips, on the general loop, then finish last) 253.5 / 166.8, with both copies
-    // 263.4 / 187.2.  Every kernel takes the copies except the accumulating ones (see the check at
-    // the top of this function); the batch's gain: 256-instance design map 116.6 -> 129.6 cells/s.
+    // 263.4 / 187.2.  Every kernel takes the copies except for accumulating units (see the check at the
+    // top of this function).  The copies (SPLIT: how many) have to fit the instruction cache: the
+    // batch kernel that holds the accumulating loop too does without the interior copy (its
+    // interior strips run the other), which gave 352 -> 336 ms on 48 uneven instances, and twice the
+    // interior loop unrolled made 2048^2 38 % slower.
     // An L2
     // prefetch of the rows beyond the ring (cp.async.bulk.prefetch.tensor) lost in both forms
     // (FP32 212.8 against 220.4, FP16 173.7 against 199.5, with one wave of units) and is not used.
@@ -608,13 +620,13 @@ __device__ __forceinline__ bool stream_unit(const UnitCtx &u, const UnitRun &r, 
             ok = false;
             break;
         }
-    if (SPLIT && xedge) {  // (without SPLIT these loops never run: f1 = f0)
+    if (SPLIT == 1 || (SPLIT == 2 && xedge)) {  // (without SPLIT these loops never run: f1 = f0)
         for (; ok && i < f1; ++i)
             if (!row(EdgeStrip{}, i, wa, wa)) {
                 ok = false;
                 break;
             }
-    } else {
+    } else if (SPLIT == 2) {
         for (; ok && i < f1; ++i)
             if (!row(Interior{}, i, wa, wa)) {
                 ok = false;
@@ -676,7 +688,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     r.src_inc = sp[warp].inc;
     RingState R{ring, bars[warp], reinterpret_cast<float4 *>(ring + RING * LY::SLOT), 0, 0u};
     bool bad = false;
-    const bool ok = stream_unit<F16, POL, ACC, !ACC, MIX>(u, r, R, bad);
+    const bool ok = stream_unit<F16, POL, ACC, ACC ? 0 : 2, MIX>(u, r, R, bad);
     if (lane == 0 && !ok) atomicOr(a.err, kErrTimeout);
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.err, kErrUnstable);
 }
@@ -701,7 +713,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     constexpr int RING = LY::RING;
     extern __shared__ unsigned char sm_dyn[];
     __shared__ __align__(8) uint64_t bars[NW][RING];
-    __shared__ MatT<float> wtab[NW][4];  // the current unit's region table, per warp
+    __shared__ PairMat wtab[NW][3 * PAIR_IDS];  // the current unit's region pairs, per warp
     __shared__ UnitCtx uctx[NW];         // the current instance, per warp (read from here, not kept in registers)
     __shared__ UnitRun urun[NW];         // the current unit, per warp
     __shared__ SrcLevels sp[NW];         // its source values (first strip), per warp
@@ -724,7 +736,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
         if (t >= steps) continue;  // uniform over the warp, like acc
         const bool acc = ACC && t + BT - 1 >= I.acc_from;
         __syncwarp();              // the previous unit's reads of the table and context are done
-        if (lane < 3) wtab[warp][lane] = I.m[lane];
+        if (lane < 9) wtab[warp][lane / 3 * PAIR_IDS + lane % 3] = pair_mat(I.m[lane % 3], I.m[lane / 3]);
         UnitCtx &u = uctx[warp];
         if (lane == 0) {
             u.nx = I.nx;
@@ -754,7 +766,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
             r.imap = maps + 3 * un.x + 2;
             tmap_acquire(r.smap);  // lane 0 issues every row copy of the unit
             tmap_acquire(r.imap);
-            r.table = wtab[warp];
+            r.pairs = wtab[warp];
             r.src_g = sp[warp].g;
             r.src_inc = sp[warp].inc;
         }
@@ -763,9 +775,9 @@ __global__ void __launch_bounds__(NW * 32, 3)
         bool bad = false;
         bool ok;
         if (ACC && acc)
-            ok = stream_unit<false, POL, true, false>(u, r, R, bad);
+            ok = stream_unit<false, POL, true, 0, false, true>(u, r, R, bad);
         else
-            ok = stream_unit<false, POL, false, true>(u, r, R, bad);
+            ok = stream_unit<false, POL, false, ACC ? 1 : 2, false, true>(u, r, R, bad);
         if (!ok) {  // a row copy never completed: report, leave
             if (lane == 0) atomicOr(err + un.x, kErrTimeout);
             return;
