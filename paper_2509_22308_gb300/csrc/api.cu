@@ -655,17 +655,16 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
     // three steps per launch (28 x 12 tiles): forced by the flag only; the four-step kernel
     // replaced it as the default on large lattices
     h->t3 = (g->flags & LBM_EM_FLAG_THREE_STEP) != 0;
-    // four steps per launch (row-streaming kernel): forced by the flag, else the default of FP32
-    // and FP16-deviation from 2^20 sites on (measured on GB300, GLUPS four / two steps per
-    // launch, FP32: 8192^2 267.9 / 136.8, 4096^2 241.5 / 138.0, 2048^2 193.1 / 122.4, 1448^2
-    // 184.4 / 114.3, 1024^2 135.0 / 117.4, 768^2 76.7 / 100.8, 512^2 34.6 / 70.4; FP16-deviation:
-    // 8192^2 277.7 / 116.8, 2048^2 197.7 / 106.9, 1448^2 171.3 / 100.2, 1024^2 127.8 / 99.2,
-    // 768^2 67.7 / 86.5, 512^2 31.0 / 59.2; three steps per launch never led: 8192^2 143.9,
-    // 1024^2 111.1: on small lattices the strips cannot fill the GPU and the two-step kernel's
-    // state stays in L2)
+    // four steps per launch (row-streaming kernel): forced by the flag, else the default of FP32 from 2^19
+    // sites on and of FP16-deviation from 2^20 (measured on GB300, us per step four / two steps per
+    // launch, FP32: 640^2 5.3 / 4.9, 700^2 5.3 / 5.3, 768^2 5.6 / 5.8, 900 x 800 6.4 / 6.7, 1024^2
+    // 7.4 / 8.8, 1536^2 12.1 / 20.3, 300 x 2000 6.0 / 6.2; GLUPS at 8192^2 267.9 / 136.8;
+    // FP16-deviation, whose bits depend on the steps per launch: GLUPS 8192^2 277.7 / 116.8, 1024^2
+    // 135 / 99; three steps per launch never led: FP32 8192^2 143.9, 1024^2 111.1 GLUPS: on small
+    // lattices the strips cannot fill the GPU and the two-step kernel's state stays in L2)
     h->s4 = (g->flags & LBM_EM_FLAG_FOUR_STEP) != 0 ||
             (!step_flags && (g->precision == LBM_EM_F32 || g->precision == LBM_EM_F16DEV) &&
-             (long long)g->nx * g->ny >= (1LL << 20));
+             (long long)g->nx * g->ny >= (g->precision == LBM_EM_F32 ? 1LL << 19 : 1LL << 20));
     if (h->s4) {
         h->t3 = false;
         h->tb = true;

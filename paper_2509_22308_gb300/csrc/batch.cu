@@ -433,9 +433,10 @@ __host__ __device__ inline int count_units(int nx, int ny, int seg) {
 // height the autotuner chose for the full batch.  A unit lasts as long as its rows and 8 halo
 // rows (about 1 us each), however idle the GPU is, so short segments are the faster ones once
 // the instances that still run leave warps idle; with every warp busy the long ones are, whose
-// halo rows cost less.  16 rows at least: shorter ones spend most of their time on the halo.
-// seg[0] = 0: no four-step launches.
-constexpr int kUnitLevels = 5;
+// halo rows cost less.
+// (us per step with 16 rows at least / 5: 6 instances of 200^2 7.3 / 5.4, 20 of 136^2 8.1 / 6.2, where two
+// steps per launch take 6.5 and 7.5.)  seg[0] = 0: no four-step launches.
+constexpr int kUnitLevels = 8;
 struct UnitPlan {
     int seg[kUnitLevels], warps;
     int4 *units;  // instance, strip, rows from .. to - 1
@@ -574,9 +575,8 @@ struct lbm_em_batch {
     TileCtx *d_ctx = nullptr;       // FP32: one record per tile of the tile list
     SrcPairF *d_srcs = nullptr;     // FP32: per instance, the source values of the current launch
     int two_ctas[3] = {0, 0, 0};
-    // four steps per launch (FP32, fixed run lengths): row-streaming kernel over work units
-    // (instance, strip, row segment of at most four_seg rows), per-instance records, tensor maps and
-    // source parameters, and the source values of the current launch
+    // four steps per launch (FP32): row-streaming kernel over work units (instance, strip, row segment of
+    // at most four_seg rows), per-instance records, tensor maps and source parameters
     bool four = false;
     UnitPlan units{};
     int four_seg = 0, four_grid = 0, four_blocks = 0, four_ctas = 0, n_units = 0;
@@ -703,7 +703,7 @@ static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
         for (int q = 0; q < 3; ++q) r.m[q] = d.mtabf[q];
     }
     UnitPlan &u = b->units;
-    u = UnitPlan{{seg, 48, 32, 24, 16}, b->four_grid * kStreamWarps, nullptr, nullptr};
+    u = UnitPlan{{seg, 48, 32, 24, 16, 12, 8, 5}, b->four_grid * kStreamWarps, nullptr, nullptr};
     b->n_units = 0;
     for (const InstDesc &d : b->desc) b->n_units += count_units(d.nx, d.ny, seg);
     const int room = std::max(b->n_units, u.warps);
@@ -914,7 +914,14 @@ static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int
     const bool pinned = want_w || want_h || want_c;
     const bool multi = b->prec == LBM_EM_F32 && b->conv_tol <= 0.0;
     if ((multi || (b->prec == LBM_EM_F32 && conv_four(b))) && b->four_grid > 0 && ((b->want_spl == 0 && !pinned) || b->want_spl == 4))
-        for (int seg : {64, 128, 256}) cands.push_back(Cand{64, 4, 4, 4, seg});
+        for (int seg : {64, 128, 256}) {
+            // only where the segments differ: not with warps left idle (UnitPlan), nor beyond every lattice's height
+            long long units = 0;
+            int tallest = 0;
+            for (const InstDesc &d : b->desc) units += count_units(d.nx, d.ny, 48), tallest = std::max(tallest, d.ny);
+            if (seg > 64 && (units <= b->four_grid * kStreamWarps || seg >= 2 * tallest)) continue;
+            cands.push_back(Cand{64, 4, 4, 4, seg});
+        }
     const int two_shapes[3][2] = {{GeoWide::KW, GeoWide::KH}, {GeoTall::KW, GeoTall::KH}, {GeoMid::KW, GeoMid::KH}};
     for (int g = 0; g < 3; ++g) {
         const int w = two_shapes[g][0], h = two_shapes[g][1], c = b->two_ctas[g];
@@ -959,16 +966,44 @@ static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int
         if (st) break;
         st = batch_clear(b);
         if (st) break;
+        // from a time in the middle of the runs, when the source's ramp is over: its evaluation is ahead of
+        // every two-step launch and made those 17 % slower there (20 instances of 64^2), four steps the choice
+        const long long mid = std::max(0LL, b->first_acc - 64), at[2] = {mid, mid};
+        st = cuda_status(copy_async(b->d_time, at, sizeof(at), cudaMemcpyHostToDevice, b->stream), "trial time");
+        if (st) break;
         const int launches = trial / c.spl;
-        cudaError_t e = batch_launch(b, b->stream, 0);  // warm-up
+        cudaError_t e = batch_launch(b, b->stream, 0, false);  // warm-up
         cudaEventRecord(e0, b->stream);
-        for (int k = 1; k <= launches && e == cudaSuccess; ++k) e = batch_launch(b, b->stream, k & 1);
+        for (int k = 1; k <= launches && e == cudaSuccess; ++k) e = batch_launch(b, b->stream, k & 1, false);
         cudaEventRecord(e1, b->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         st = cuda_status(e, "autotune launch");
         if (st) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
+        if (c.spl > 1 && ms < 0.06f * launches) {
+            // short launches: timed again as the run replays them, for the host's pace and the gaps between
+            // kernels decided there (6 instances of 200^2 took 16-row units, four steps per launch, where
+            // two were 13 % faster)
+            st = batch_capture(b, launches & 1 ? 0 : 1, false);
+            if (st) break;
+            cudaGraphExec_t &g = b->graph[launches & 1 ? 0 : 1][0];
+            for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, b->stream);
+            cudaEventRecord(e0, b->stream);
+            for (int k = 0; k < 2 * launches && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, b->stream);
+            cudaEventRecord(e1, b->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+            st = cuda_status(e, "autotune launch");
+            if (st) break;
+            cudaEventElapsedTime(&ms, e0, e1);
+            ms *= 0.25f;  // a graph holds two launches
+        }
+        // row segments: the shortest are timed first, and longer ones have to win clearly, because
+        // later in a run, when instances have stopped or accumulate, the shorter ones gain (48 uneven
+        // instances: a trial even within 1 %, the run 352 ms with 64 rows and 378 with 128)
+        if (c.spl == 4 && c.seg > 64) ms *= 1.03f;
         if (ms < best) {
             best = ms;
             bc = c;

@@ -870,8 +870,11 @@ StreamPlan stream_plan(int nx, int ny, int resident_warps, bool f16) {
         if (k > 1 && (ny + sk - 1) / sk < min_rows) break;
         segs = sk;
     }
-    // but at least 16 rows each (shorter ones spend most of their time on the halo)
-    if (segs > (ny + 15) / 16) segs = (ny + 15) / 16;
+    // but at least 5 rows each.  Where a wave of longer segments leaves warps idle, a launch lasts as
+    // long as one unit, its rows and 8 halo rows (us per step with at least 16 / 8 / 5 rows: FP32 768^2
+    // 7.4 / 6.3 / 5.6, 900 x 800 7.4 / 6.4 / 6.4, 1200 x 1100 9.3 / 8.7 / 8.7; FP16-deviation 1200 x 1100
+    // 9.7 / 9.0 / 9.0)
+    if (segs > (ny + 4) / 5) segs = (ny + 4) / 5;
     p.seg_rows = (ny + segs - 1) / segs;
     segs = (ny + p.seg_rows - 1) / p.seg_rows;
     p.n_units = p.n_strips * segs;
