@@ -78,10 +78,13 @@ typedef enum {
 } lbm_em_source_kind;
 
 /* lbm_em_grid.flags: how many time steps one kernel launch advances.  By default FP64 and
- * double-float advance one step per launch; FP32 and FP16-deviation two below 2^20 sites
- * (each tile and its halo are copied to shared memory by the TMA unit and advance two
+ * double-float advance one step per launch; FP32 two below 2^19 sites and FP16-deviation below
+ * 2^20 (each tile and its halo are copied to shared memory by the TMA unit and advance two
  * steps there), four from there on (each warp streams a strip of the lattice through four time
- * levels held in registers).  The flags force a mode.  In FP32, FP64 and double-float the
+ * levels held in registers).  Runs of FP64, FP32 and double-float lattices small enough to stay
+ * on chip (about 550^2, 600^2 and 350^2 sites) take up to 256 steps in one cooperative launch
+ * instead: FP32 from 330^2 sites on always, the others on the library's own stream while no
+ * other such handle has steps in flight.  The flags force a mode and rule that out.  In FP32, FP64 and double-float the
  * result does not depend on the choice: every mode gives the same bits.  In FP16-deviation the
  * four-step mode rounds the stored state to FP16 once per launch instead of once per step, so
  * its bits differ from the other modes by FP16 rounding noise (its runs still give the same
