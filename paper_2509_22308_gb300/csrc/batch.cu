@@ -988,9 +988,9 @@ static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int
             st = batch_capture(b, launches & 1 ? 0 : 1, false);
             if (st) break;
             cudaGraphExec_t &g = b->graph[launches & 1 ? 0 : 1][0];
-            for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, b->stream);
+            e = cudaGraphLaunch(g, b->stream);
             cudaEventRecord(e0, b->stream);
-            for (int k = 0; k < 2 * launches && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, b->stream);
+            for (int k = 0; k < launches && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, b->stream);
             cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             cudaGraphExecDestroy(g);
@@ -998,7 +998,7 @@ static lbm_em_status batch_autotune(lbm_em_batch *b, int want_w, int want_h, int
             st = cuda_status(e, "autotune launch");
             if (st) break;
             cudaEventElapsedTime(&ms, e0, e1);
-            ms *= 0.25f;  // a graph holds two launches
+            ms *= 0.5f;  // a graph holds two launches
         }
         // row segments: the shortest are timed first, and longer ones have to win clearly, because
         // later in a run, when instances have stopped or accumulate, the shorter ones gain (48 uneven
