@@ -67,18 +67,10 @@ __device__ __forceinline__ T from_left(T v, T in, int lane) {
     const T l = shfl_from(v, -1);
     return lane == 0 ? in : l;
 }
-__device__ __forceinline__ f2 from_left(f2 v, float in, int lane) {
-    const float l = shfl_from(hi2(v), -1);
-    return pack2(lane == 0 ? in : l, lo2(v));
-}
 template <typename T>
 __device__ __forceinline__ T from_right(T v, T in, int lane) {
     const T r = shfl_from(v, 1);
     return lane == 31 ? in : r;
-}
-__device__ __forceinline__ f2 from_right(f2 v, float in, int lane) {
-    const float r = shfl_from(lo2(v), 1);
-    return pack2(hi2(v), lane == 31 ? in : r);
 }
 // The lattice's last column keeps its own value (zero-gradient open edge).
 template <typename T>
@@ -129,13 +121,10 @@ __device__ __forceinline__ void msg_store(Msg *p, unsigned long long v, unsigned
 }
 __device__ __forceinline__ unsigned long long word_of(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ unsigned long long word_of(df v) { return pack2(v.hi, v.lo).v; }
-__device__ __forceinline__ unsigned long long word_of(f2 v) { return v.v; }
 __device__ __forceinline__ void from_word(unsigned long long w, double &v) { v = __longlong_as_double((long long)w); }
 __device__ __forceinline__ void from_word(unsigned long long w, df &v) { v = df(lo2(f2{w}), hi2(f2{w})); }
-__device__ __forceinline__ void from_word(unsigned long long w, f2 &v) { v.v = w; }
 
 // The two values of a border site (p[0 .. MSGS - 1]).
-__device__ __forceinline__ void send_site(Msg *p, float a, float b, unsigned seq) { msg_store(p, pack2(a, b).v, seq); }
 template <typename T>
 __device__ __forceinline__ void send_site(Msg *p, T a, T b, unsigned seq) {
     msg_store(p, word_of(a), seq);
@@ -162,7 +151,6 @@ __device__ __forceinline__ Msg msg_get(const Msg *p) {
                  : "memory");
     return m;
 }
-__device__ __forceinline__ void put_site(Msg *p, float a, float b, unsigned seq) { msg_put(p, pack2(a, b).v, seq); }
 template <typename T>
 __device__ __forceinline__ void put_site(Msg *p, T a, T b, unsigned seq) {
     msg_put(p, word_of(a), seq);
