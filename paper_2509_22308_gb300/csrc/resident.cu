@@ -802,7 +802,8 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     auto receive = [&](const RowLink<V> &l, int k, V &v, V &h) -> bool {
         Patience pt;
         if (l.here) {
-            while ((int)(flag_get(l.flag) - (unsigned)k) < 0)
+            // by a vote, like every wait here: over() needs all lanes, and each lane's own acquire orders its reads
+            while (!__all_sync(kFull, (int)(flag_get(l.flag) - (unsigned)k) >= 0))
                 if (pt.over(a.err)) return false;
             const V *const q = l.buf + ((k + 1) & 1) * bstep;
             v = q[0];
