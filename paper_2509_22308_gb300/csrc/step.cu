@@ -105,7 +105,8 @@ template <typename T>
 cudaError_t launch_step(const StepArgs<T> &a, const T *fin, T *fout, const long long *t_in,
                         long long *t_out, bool accumulate, cudaStream_t s) {
     if constexpr (std::is_same<T, df>::value)
-        if (!accumulate) {
+        // beyond 65535 of its blocks along y (4 rows each) the scalar kernel's (8 rows each) still fit
+        if (!accumulate && (a.ny + 2 * DFY - 1) / (2 * DFY) <= 65535) {
             const dim3 grid((a.nx + BX - 1) / BX, (a.ny + 2 * DFY - 1) / (2 * DFY)), block(BX, DFY);
             if (a.pol == POL_TE)
                 k_step_df<POL_TE><<<grid, block, 0, s>>>(a, fin, fout, t_in, t_out);
