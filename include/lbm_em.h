@@ -181,7 +181,8 @@ lbm_em_status lbm_em_step(lbm_em_t *h, int64_t n);
 
 /* Wait for the handle's stream; returns LBM_EM_EUNSTABLE if any step flagged a
  * non-finite or runaway field since creation (the flag is sticky), LBM_EM_ETIMEOUT if a
- * tile copy of a step never completed.  After LBM_EM_ETIMEOUT a copy may still have been in
+ * tile copy of a step never completed or, in a launch of many steps, a neighbouring thread
+ * block's message never came.  After LBM_EM_ETIMEOUT a copy may still have been in
  * flight when its thread block left, so the handle's state is undefined: lbm_em_step and
  * lbm_em_accumulate then return LBM_EM_ESTATE, and the handle must be destroyed. */
 lbm_em_status lbm_em_sync(lbm_em_t *h);
@@ -273,6 +274,15 @@ const char *lbm_em_last_error(void);
  * reported: LBM_EM_ETIMEOUT is the expected result; the device stays usable.  Synchronous,
  * on the legacy default stream; LBM_EM_EINVAL for a limit outside the range. */
 lbm_em_status lbm_em_probe_bounded_wait(int64_t limit_cycles);
+
+/* Fault injection for tests of the waits between thread blocks (the paper has no counterpart).
+ * From now on h's launches of many steps (lbm_em_grid.flags) leave out their last thread
+ * block, whose messages the others then wait for, and every wait gives up after limit_cycles
+ * (1 .. 2e9) clock cycles instead of about 2e9: the next such run ends by itself, and
+ * lbm_em_sync returns LBM_EM_ETIMEOUT.  Nothing faults and the device stays usable; the handle
+ * must be destroyed.  LBM_EM_EINVAL for a limit outside the range, LBM_EM_ESTATE if the handle
+ * takes no such launches or only ones of one block. */
+lbm_em_status lbm_em_test_lost_messages(lbm_em_t *h, int64_t limit_cycles);
 
 /* Diagnostic of the FP64 pipe (the paper has no counterpart), the ceiling of the FP64 step on
  * GB300: enqueues on `stream` (a cudaStream_t; NULL: the legacy default stream) one launch of

@@ -20,6 +20,7 @@
 #include "runtime.h"
 #include "step2.cuh"
 #include "step2_tma.h"
+#include "tma.cuh"
 #include "step_f16.cuh"
 #include "step_stream.h"
 
@@ -958,9 +959,19 @@ lbm_em_status lbm_em_sync(lbm_em_t *h) {
     if (st) return st;
     if (err & kErrTimeout) {
         h->timed_out = true;
-        return set_error(LBM_EM_ETIMEOUT, "a bounded wait for a tile load gave up");
+        return set_error(LBM_EM_ETIMEOUT, "a bounded wait for a tile load or a neighbouring block's message gave up");
     }
     if (err) return set_error(LBM_EM_EUNSTABLE, "a field became non-finite or exceeded 3 * 2^20 times the source amplitude");
+    return LBM_EM_OK;
+}
+
+lbm_em_status lbm_em_test_lost_messages(lbm_em_t *h, int64_t limit_cycles) {
+    if (!h) return set_error(LBM_EM_EINVAL, "handle is NULL");
+    if (limit_cycles < 1 || limit_cycles > kWaitCycles)
+        return set_error(LBM_EM_EINVAL, "limit_cycles must be in 1 .. 2e9");
+    if (h->res.ctas < 2) return set_error(LBM_EM_ESTATE, "no thread blocks of this handle send each other messages");
+    h->res.launch = h->res.ctas - 1;
+    h->res.wait = limit_cycles;
     return LBM_EM_OK;
 }
 

@@ -18,8 +18,8 @@
 // A mailbox has two slots, used in turn: a sender overwrites a message after it has received the
 // neighbour's following one, which the neighbour sent when it had read it.  Sequence numbers go on
 // from launch to launch (a device word), so an old message is never taken for a new one.  Every wait
-// is bounded (kWaitCycles) and reports kErrTimeout; the cooperative launch guarantees that all the
-// blocks run at the same time.
+// is bounded (ResidentPlan::wait) and a warp that gives up reports kErrTimeout, which ends the others';
+// the cooperative launch guarantees that all the blocks run at the same time.
 //
 // The per-site arithmetic is the one-step kernel's (moments / collide, update_pair for FP32), so every
 // form gives the bits of one step per launch.  Accumulating launches store the fields of the
@@ -214,7 +214,8 @@ struct ResidentArgs {
     T *fout;
     const long long *t_in;
     long long *t_out;
-    int strips, rows, segs, warps, comm, total, n;
+    int strips, rows, segs, warps, comm, total, ctas, n;
+    long long wait;   // clock cycles after which a wait gives up
     Msg *xm, *ym;
     unsigned *ctl;    // [0]: sequence number of the launch's start, [1]: blocks that have finished
     T *stage;
@@ -250,14 +251,16 @@ __device__ __forceinline__ unsigned flag_get(const unsigned *f) {
     return v;
 }
 
-// Up to kWaitCycles of failed attempts; true: give up (also once another block has).
+// Up to r.wait clock cycles of failed attempts; true: give up (also once another warp has).  All lanes of
+// the warp call it together.
 struct Patience {
     long long c0 = 0;
     unsigned spin = 0;
-    __device__ __forceinline__ bool over(const unsigned *err) {
+    template <typename T>
+    __device__ __forceinline__ bool over(const ResidentArgs<T> &r) {
         if (++spin == 1) c0 = clock64();
         if (spin & 63u) return false;
-        return __any_sync(kFull, clock64() - c0 > kWaitCycles || (*(const volatile unsigned *)err & kErrTimeout));
+        return __any_sync(kFull, clock64() - c0 > r.wait || (*(const volatile unsigned *)r.a.err & kErrTimeout));
     }
 };
 
@@ -285,7 +288,7 @@ __device__ void watch_mail(const ResidentArgs<T> &r, unsigned base, int cw, int 
     constexpr int MSGS = Form<T>::MSGS;
     const int ny = r.a.ny, first = (int)blockIdx.x * r.warps, warps = min(r.warps, r.total - first);
     const int n_x = warps * r.rows * 2 * MSGS;
-    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * MSGS, yslot = (size_t)gridDim.x * 2 * 64;
+    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * MSGS, yslot = (size_t)r.ctas * 2 * 64;
     const Msg *src[kWatch];
     Msg *dst[kWatch];
     unsigned left[kWatch];  // messages still to come
@@ -337,7 +340,7 @@ __device__ void watch_mail(const ResidentArgs<T> &r, unsigned base, int cw, int 
         }
         if (__any_sync(kFull, got)) {
             pt.spin = 0;
-        } else if (pt.over(r.a.err)) {
+        } else if (pt.over(r)) {
             if (lane == 0) atomicOr(r.a.err, kErrTimeout);
             return;
         }
@@ -607,7 +610,9 @@ __global__ void __launch_bounds__(resident32_warps(R) * 32, 1)
                     if (has_down && y >= yo1 - H) send_pair(ym + (b * 2 * H + (y - ynext)) * kHaloMsgs * np + xa / 2, np, st[i], seq);
                 }
             }
-            // a row's eight messages are in flight together (two rows' at once gained nothing)
+            // a row's eight messages are in flight together (two rows' at once gained nothing); the rows share
+            // one limit, so that a warp that gives up does so after one wait, not after one per row
+            Patience pt;
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 const int y = y0 + i;
@@ -622,7 +627,6 @@ __global__ void __launch_bounds__(resident32_warps(R) * 32, 1)
                         src = ym + (b * 2 * H + (y - ynext)) * kHaloMsgs * np + xa / 2;
                 }
                 bool need = src != nullptr;
-                Patience pt;
                 while (__any_sync(kFull, need)) {
                     if (need) {
                         Msg v[kHaloMsgs];
@@ -633,7 +637,7 @@ __global__ void __launch_bounds__(resident32_warps(R) * 32, 1)
                             need = false;
                         }
                     }
-                    if (pt.over(a.err)) {
+                    if (pt.over(r)) {
                         ok = false;
                         break;
                     }
@@ -745,7 +749,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     // mailboxes: xm[slot][strip border][0: going right, 1: going left][row][message],
     // ym[slot][receiving block][0: from above, 1: from below][message][lane]; inboxes:
     // xin[slot][warp][row][0: from the left, 1: from the right][message], yin[slot][0, 1][message][lane]
-    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * F::MSGS, yslot = (size_t)gridDim.x * 2 * 64;
+    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * F::MSGS, yslot = (size_t)r.ctas * 2 * 64;
     const int xin_slot = r.warps * r.rows * 2 * F::MSGS;
     Msg *const xin = reinterpret_cast<Msg *>(sm + o.xin), *const yin = reinterpret_cast<Msg *>(sm + o.yin);
     Msg *const my_xin = xin + loc * r.rows * 2 * F::MSGS;
@@ -804,7 +808,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         if (l.here) {
             // by a vote, like every wait here: over() needs all lanes, and each lane's own acquire orders its reads
             while (!__all_sync(kFull, (int)(flag_get(l.flag) - (unsigned)k) >= 0))
-                if (pt.over(a.err)) return false;
+                if (pt.over(r)) return false;
             const V *const q = l.buf + ((k + 1) & 1) * bstep;
             v = q[0];
             h = q[32];
@@ -813,7 +817,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         const unsigned seq = base + (unsigned)k;
         const Msg *const q = l.box + (seq & 1u) * 128;
         while (!__all_sync(kFull, get_row(q, v, h, seq)))
-            if (pt.over(a.err)) return false;
+            if (pt.over(r)) return false;
         return true;
     };
 
@@ -855,7 +859,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                     const Msg *const xr = my_xin + (seq & 1u) * xin_slot + (i * 2 + (lane == 0 ? 0 : 1)) * F::MSGS;
                     Patience pt;
                     while (!__all_sync(kFull, !waits_x || get_site<T>(xr, in0, in1, seq)))
-                        if (pt.over(a.err)) return false;
+                        if (pt.over(r)) return false;
                 }
                 const V epx = w[P_EPX * 32], emx = w[P_EMX * 32], hxpx = w[P_HXPX * 32], hxmx = w[P_HXMX * 32];
                 p.ez = w[P_EZ * 32];
@@ -1111,6 +1115,8 @@ cudaError_t resident_plan(int nx, int ny, ResidentPlan *plan) {
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, (p.warps + p.comm) * 32, p.smem);
         if (e == cudaSuccess && per_sm < 1) return cudaSuccess;
     }
+    p.wait = kWaitCycles;
+    p.launch = p.ctas;
     if (e == cudaSuccess) *plan = p;
     return e;
 }
@@ -1131,14 +1137,16 @@ cudaError_t launch_resident(const StepArgs<T> &a, const T *fin, T *fout, const l
     r.warps = plan.warps;
     r.comm = plan.comm;
     r.total = plan.total;
+    r.ctas = plan.ctas;
     r.n = n;
+    r.wait = plan.wait;
     r.xm = (Msg *)mail;
     r.ym = r.xm + 2 * plan.mail_x;
     r.ctl = ctl;
     r.stage = stage;
     r.n_slots = n_slots;
     void *args[] = {&r};
-    cudaError_t e = cudaLaunchCooperativeKernel(kernel_of<T>(a.pol, accumulate, plan.rows), dim3(plan.ctas), dim3((plan.warps + plan.comm) * 32),
+    cudaError_t e = cudaLaunchCooperativeKernel(kernel_of<T>(a.pol, accumulate, plan.rows), dim3(plan.launch), dim3((plan.warps + plan.comm) * 32),
                                                 args, plan.smem, s);
     if (e == cudaSuccess && accumulate && n_slots > 0) {
         k_resident_flush<T><<<(6 * n_slots + 31) / 32, 32, 0, s>>>(stage, a.accp.acc, n_slots, n, a.src.cs, a.src.period,

@@ -15,8 +15,11 @@ constexpr int kResidentHalo = 4;  // FP32: steps between two exchanges of the ti
 // How a lattice is spread over the GPU: strips of 32 lanes (64 columns in FP32, 32 in the 8-byte
 // forms) cut into segments of `rows` rows, one warp each; `warps` such warps and
 // `comm` communication warps per thread block, at most one block per SM.  ctas == 0: the lattice does not fit (or is better off elsewhere).
+// wait: clock cycles after which a wait for another block or warp gives up; launch: the blocks that are
+// launched, all of them except in a test of those waits.
 struct ResidentPlan {
-    int ctas, strips, rows, segs, warps, comm, total;
+    int ctas, strips, rows, segs, warps, comm, total, launch;
+    long long wait;
     size_t smem, mail_x, mail_bytes;
 };
 

@@ -97,6 +97,7 @@ SIGNATURES = {
     "lbm_em_rasterize_janus": [_P(Janus), ctypes.c_int32, ctypes.c_int32, _P(ctypes.c_uint8)],
     "lbm_em_rasterize_janus_noalloc": [_P(Janus), ctypes.c_int32, ctypes.c_int32, _P(ctypes.c_uint8)],
     "lbm_em_probe_bounded_wait": [ctypes.c_int64],
+    "lbm_em_test_lost_messages": [_vp, ctypes.c_int64],
     "lbm_em_test_alloc_hook": [ctypes.c_int64, _P(ctypes.c_int64)],
     "lbm_em_probe_fp64_fma": [_vp, ctypes.c_int64, _P(ctypes.c_double)],
     "lbm_em_probe_f16_rebuild": [_P(ctypes.c_uint32), _P(ctypes.c_float), ctypes.c_int64, ctypes.c_int32,
@@ -238,6 +239,11 @@ class Solver:
         v = ctypes.c_int32()
         _call("lbm_em_get_steps_per_launch", self.h, ctypes.byref(v))
         return v.value
+
+    def lose_messages(self, limit_cycles):
+        """Test hook: the handle's launches of many steps leave out a thread block and give up waiting for its
+        messages after ``limit_cycles`` clock cycles (``lbm_em_test_lost_messages``)."""
+        _call("lbm_em_test_lost_messages", self.h, ctypes.c_int64(int(limit_cycles)))
 
     def set_contour(self, c: Contour):
         _call("lbm_em_set_contour", self.h, ctypes.byref(c))
