@@ -187,11 +187,16 @@ lbm_em_status lbm_em_step(lbm_em_t *h, int64_t n);
  * lbm_em_accumulate then return LBM_EM_ESTATE, and the handle must be destroyed. */
 lbm_em_status lbm_em_sync(lbm_em_t *h);
 
-/* Time steps one launch of the handle's step kernel advances (1, 2, 3 or 4), the mode that
- * lbm_em_grid.flags forced or the default chose for the form and lattice size.  Runs of fewer
- * steps, and the steps that bring an odd start time to an even one for two-step launches,
- * take single-step launches. */
+/* Time steps one plain launch of the handle's step kernel advances (1, 2, 3 or 4), the mode
+ * that lbm_em_grid.flags forced or the default chose for the form and lattice size.  Runs of
+ * fewer steps, and the steps that bring an odd start time to an even one for two-step launches,
+ * take single-step launches.  The launches of up to 256 steps that lattices kept on chip take
+ * instead (lbm_em_grid.flags) are counted by lbm_em_get_resident_launches. */
 lbm_em_status lbm_em_get_steps_per_launch(lbm_em_t *h, int32_t *n);
+
+/* Launches of many steps with the state on chip (lbm_em_grid.flags) that the handle has enqueued
+ * since its creation; 0 for a handle whose steps have all been plain launches. */
+lbm_em_status lbm_em_get_resident_launches(lbm_em_t *h, int64_t *n);
 
 /* Current time step count (host view; equals the number of steps enqueued). */
 lbm_em_status lbm_em_get_time(lbm_em_t *h, int64_t *t);

@@ -242,6 +242,7 @@ struct lbm_em {
     ResidentPlan res{};
     void *d_mail = nullptr;
     unsigned *d_ctl = nullptr;
+    int64_t res_launches = 0;        // enqueued so far
     bool res_shares = false;         // resident only while no other such handle has steps in flight (others_busy)
     bool busy = false;               // res_shares: busy_ev marks the end of the steps enqueued last
     cudaEvent_t busy_ev = nullptr;
@@ -513,6 +514,7 @@ static lbm_em_status run_steps(lbm_em *h, int64_t n, bool acc) {
                 break;
             }
             if (lbm_em_status st = cuda_status(e, "resident step launch")) return st;
+            ++h->res_launches;
             h->cur ^= 1;
             h->t += c;
             n -= c;
@@ -978,6 +980,12 @@ lbm_em_status lbm_em_test_lost_messages(lbm_em_t *h, int64_t limit_cycles) {
 lbm_em_status lbm_em_get_steps_per_launch(lbm_em_t *h, int32_t *n) {
     if (!h || !n) return set_error(LBM_EM_EINVAL, "NULL argument");
     *n = launch_steps(h, false);
+    return LBM_EM_OK;
+}
+
+lbm_em_status lbm_em_get_resident_launches(lbm_em_t *h, int64_t *n) {
+    if (!h || !n) return set_error(LBM_EM_EINVAL, "NULL argument");
+    *n = h->res_launches;
     return LBM_EM_OK;
 }
 

@@ -79,6 +79,7 @@ SIGNATURES = {
     "lbm_em_sync": [_vp],
     "lbm_em_get_time": [_vp, _P(ctypes.c_int64)],
     "lbm_em_get_steps_per_launch": [_vp, _P(ctypes.c_int32)],
+    "lbm_em_get_resident_launches": [_vp, _P(ctypes.c_int64)],
     "lbm_em_set_contour": [_vp, _P(Contour)],
     "lbm_em_accumulate": [_vp, ctypes.c_int64],
     "lbm_em_contour_integral": [_vp, _P(ctypes.c_double)],
@@ -238,6 +239,12 @@ class Solver:
     def steps_per_launch(self) -> int:
         v = ctypes.c_int32()
         _call("lbm_em_get_steps_per_launch", self.h, ctypes.byref(v))
+        return v.value
+
+    def resident_launches(self) -> int:
+        """Launches of many steps with the state on chip that the handle has enqueued so far."""
+        v = ctypes.c_int64()
+        _call("lbm_em_get_resident_launches", self.h, ctypes.byref(v))
         return v.value
 
     def lose_messages(self, limit_cycles):
