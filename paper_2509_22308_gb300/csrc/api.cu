@@ -604,6 +604,31 @@ static std::vector<MatT<T>> material_table(const double *eps, const bool *pec) {
     return tab;
 }
 
+// Whether four steps per launch (row-streaming kernel) are the default of a form and lattice size: of
+// FP16-deviation and FP32 from 2^20 sites on, and of FP32 below that from 2^19 sites on where the strips
+// are well filled (measured on GB300, us per step four / two steps per launch, FP32: 640^2 5.3 / 4.9,
+// 700^2 5.3 / 5.3, 768^2 5.6 / 5.8, 900 x 800 6.4 / 6.7, 1024^2 7.4 / 8.8, 1536^2 12.1 / 20.3; GLUPS at
+// 8192^2 267.9 / 136.8; FP16-deviation, whose bits depend on the steps per launch: GLUPS 8192^2 277.7
+// / 116.8, 1024^2 135 / 99; three steps per launch never led: FP32 8192^2 143.9, 1024^2 111.1 GLUPS:
+// on small lattices the strips cannot fill the GPU and the two-step kernel's state stays in L2).
+// A strip yields 56 columns and a tile of the two-step kernel is 64 x 8, so a narrow lattice can need up to
+// twice as many strips as tiles along x, and then takes four steps per launch only when its tiles cover
+// more (us per step four / two at about 530, 750 and 1040 thousand sites by width, strips / tiles: 100
+// (1.0) 5.7 / 6.3, 6.8 / 8.3, 8.1 / 13.7; 400 (1.14) 5.7 / 5.9, 6.8 / 7.5, 7.9 / 9.5; 320 (1.2) 5.7 / 5.4, 6.4 /
+// 6.7, 7.6 / 8.7; 256 (1.25) 5.6 / 5.5, 6.7 / 6.6, 7.8 / 8.7; 192 (1.33) 6.0 / 5.5, 6.7 / 6.6, 7.9 / 8.7; 128 (1.5)
+// 6.1 / 5.4, 7.1 / 6.6, 8.6 / 8.8; 64 (2) 7.2 / 5.6, 8.2 / 6.5, 10.1 / 8.8): the covered sites from which it leads
+// grow as the square of that ratio.  A state of more than about 95 MB leaves the two-step kernel's L2
+// (60 x 17333, rows of 64: 10.7 / 11.4).
+static bool four_by_default(int precision, long long nx, long long ny) {
+    const long long sites = nx * ny;
+    if (precision != LBM_EM_F32) return precision == LBM_EM_F16DEV && sites >= 1LL << 20;
+    if (sites < 1LL << 19) return false;
+    if (sites >= 1LL << 20 || 20 * round_up((int)nx, 32) * ny >= 21LL << 20) return true;
+    const long long strips = (nx + kStreamOutW - 1) / kStreamOutW, tiles = (nx + kTmaTileW - 1) / kTmaTileW;
+    const long long covered = tiles * kTmaTileW * round_up((int)ny, kTmaTileH);
+    return covered * tiles * tiles >= (3LL << 17) * strips * strips;
+}
+
 // Allocate and initialise everything except the material ids.
 static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s, lbm_em **out) {
     if (!g || !out) return set_error(LBM_EM_EINVAL, "grid/out is NULL");
@@ -658,16 +683,9 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
     // three steps per launch (28 x 12 tiles): forced by the flag only; the four-step kernel
     // replaced it as the default on large lattices
     h->t3 = (g->flags & LBM_EM_FLAG_THREE_STEP) != 0;
-    // four steps per launch (row-streaming kernel): forced by the flag, else the default of FP32 from 2^19
-    // sites on and of FP16-deviation from 2^20 (measured on GB300, us per step four / two steps per
-    // launch, FP32: 640^2 5.3 / 4.9, 700^2 5.3 / 5.3, 768^2 5.6 / 5.8, 900 x 800 6.4 / 6.7, 1024^2
-    // 7.4 / 8.8, 1536^2 12.1 / 20.3, 300 x 2000 6.0 / 6.2; GLUPS at 8192^2 267.9 / 136.8;
-    // FP16-deviation, whose bits depend on the steps per launch: GLUPS 8192^2 277.7 / 116.8, 1024^2
-    // 135 / 99; three steps per launch never led: FP32 8192^2 143.9, 1024^2 111.1 GLUPS: on small
-    // lattices the strips cannot fill the GPU and the two-step kernel's state stays in L2)
+    // four steps per launch: forced by the flag or the default
     h->s4 = (g->flags & LBM_EM_FLAG_FOUR_STEP) != 0 ||
-            (!step_flags && (g->precision == LBM_EM_F32 || g->precision == LBM_EM_F16DEV) &&
-             (long long)g->nx * g->ny >= (g->precision == LBM_EM_F32 ? 1LL << 19 : 1LL << 20));
+            (!step_flags && four_by_default(g->precision, g->nx, g->ny));
     if (h->s4) {
         h->t3 = false;
         h->tb = true;
