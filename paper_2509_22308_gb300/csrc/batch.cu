@@ -441,6 +441,7 @@ struct UnitPlan {
     int seg[kUnitLevels], warps;
     int4 *units;  // instance, strip, rows from .. to - 1
     int *n_units;
+    long long *listed;  // the time of the last listing
 };
 
 // One block: the work units of the instances whose run goes past time t (an instance's units in a
@@ -459,6 +460,7 @@ __device__ void build_units(const InstDesc *desc, int n, long long t, const Unit
         while (k > 0 && (active[k] > u.warps || u.seg[k] >= u.seg[0])) --k;
         level = k;
         *u.n_units = active[k];
+        *u.listed = t;
         count = 0;
     }
     __syncthreads();
@@ -476,15 +478,20 @@ __global__ void __launch_bounds__(1024) k_batch_units(const InstDesc *desc, int 
     build_units(desc, n, t, u);
 }
 
-// One block: the exits of the step before *t_next, then the units of the instances that still run.
+// One block: the exits of the step before *t_next, then the units of the instances that still run, if any has
+// ended since the last listing (listing one instance of 200^2 takes longer than its one-step launch, and
+// with periods of 8 steps every second launch is followed by this kernel).
 __global__ void __launch_bounds__(1024) k_batch_converge(InstDesc *desc, StreamInst *si, double *energy, double *prev,
                                                          int *settled, const long long *__restrict__ t_next, double tol,
                                                          int min_periods, int n, const UnitPlan u) {
     const long long t = *t_next - 1;
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
+    const long long listed = u.seg[0] > 0 ? *u.listed : t + 1;
+    bool ended = false;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
         converge(desc[i], si, energy, prev, settled, t, tol, min_periods, i);
-    __syncthreads();
-    if (u.seg[0] > 0) build_units(desc, n, t + 1, u);
+        ended |= desc[i].steps > listed && desc[i].steps <= t + 1;
+    }
+    if (__syncthreads_or(ended)) build_units(desc, n, t + 1, u);
 }
 
 // Per-instance stress-tensor integral: block i reduces instance i's contour.
@@ -703,15 +710,16 @@ static lbm_em_status batch_units(lbm_em_batch *b, int seg) {
         for (int q = 0; q < 3; ++q) r.m[q] = d.mtabf[q];
     }
     UnitPlan &u = b->units;
-    u = UnitPlan{{seg, 48, 32, 24, 16, 12, 8, 5}, b->four_grid * kStreamWarps, nullptr, nullptr};
+    u = UnitPlan{{seg, 48, 32, 24, 16, 12, 8, 5}, b->four_grid * kStreamWarps, nullptr, nullptr, nullptr};
     b->n_units = 0;
     for (const InstDesc &d : b->desc) b->n_units += count_units(d.nx, d.ny, seg);
     const int room = std::max(b->n_units, u.warps);
     dfree(b->d_units);
     b->d_units = nullptr;
-    lbm_em_status st = cuda_status(dmalloc(&b->d_units, (size_t)room * sizeof(int4) + sizeof(int)), "cudaMalloc(units)");
+    lbm_em_status st = cuda_status(dmalloc(&b->d_units, (size_t)(room + 1) * sizeof(int4)), "cudaMalloc(units)");
     u.units = b->d_units;
     u.n_units = (int *)(b->d_units + room);
+    u.listed = (long long *)(b->d_units + room) + 1;
     if (!st && !b->d_sinsts)
         st = cuda_status(dmalloc(&b->d_sinsts, si.size() * sizeof(StreamInst)), "cudaMalloc(stream records)");
     if (!st)
@@ -842,10 +850,12 @@ static long long conv_gap(const lbm_em_batch *b, long long t) {
     return gap;
 }
 
-// Whether four-step launches take at least half of a convergence run's steps.  With one period P they
-// take all but one to four steps of each (180 against 57 GLUPS on 96 instances of 200^2); with many
-// different periods in one batch few gaps hold four steps, and the one-step kernel on its tuned
-// tiles is as good.
+// Whether four-step launches take at least 5/8 of a convergence run's steps.  With one period P they
+// take all but one to four steps of each (180 against 57 GLUPS on 96 instances of 200^2); with short or
+// many different periods few gaps hold four steps, and the one-step kernel replayed from a graph on
+// its tuned tiles is faster (ms one-step / four-step launches, 1 instance of 200^2 and 200 of 80^2, about
+// 480 steps: P = 8, half of the steps, 3.4 / 4.1 and 22.0 / 25.2; P = 7, 4/7, 3.7 / 4.0 and 21.9 / 23.6; P = 6 and
+// 12, 2/3, 3.8 / 3.8 and 22.0 / 21.4, 3.8 / 3.4 and 22.2 / 19.3; P = 9, 8/9, 3.7 / 2.7 and 21.8 / 13.2).
 static bool conv_four(const lbm_em_batch *b) {
     long long in4 = 0;
     for (long long t = 0; t < b->max_steps;) {
@@ -853,7 +863,7 @@ static bool conv_four(const lbm_em_batch *b) {
         in4 += gap / 4 * 4;
         t += gap;
     }
-    return 2 * in4 >= b->max_steps;
+    return 8 * in4 >= 5 * b->max_steps;
 }
 
 // Whether `n` four-step launches from time t may find an instance in its accumulated period.
