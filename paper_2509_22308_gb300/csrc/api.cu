@@ -238,11 +238,9 @@ struct lbm_em {
     bool rest2 = false;  // s4: a remainder of two or three steps takes a two-step launch (run_steps)
     CUtensorMap s4_smap[2], s4_fmap[2], s4_imap;
     StreamPlan s4_plan{}, s4_plan_acc{};  // plain and (FP32) accumulating four-step launches
-    // many steps per launch with the state on chip (small lattices, no step flag): plan, mailboxes
-    // and control words
+    // many steps per launch with the state on chip (small lattices, no step flag): plan, control words
+    // and mailboxes behind the state in buf[1]
     ResidentPlan res{};
-    void *d_mail = nullptr;
-    unsigned *d_ctl = nullptr;
     int64_t res_launches = 0;        // enqueued so far
     bool res_shares = false;         // resident only while no other such handle has steps in flight (others_busy)
     bool busy = false;               // res_shares: busy_ev marks the end of the steps enqueued last
@@ -467,7 +465,8 @@ static bool others_busy(const lbm_em *h) {
 
 static void mark_busy(lbm_em *h) {
     std::lock_guard<std::mutex> lock(g_busy_mu);
-    h->busy = cudaEventRecord(h->busy_ev, h->stream) == cudaSuccess;
+    if (!h->busy_ev && cudaEventCreateWithFlags(&h->busy_ev, cudaEventDisableTiming) != cudaSuccess) h->busy_ev = nullptr;
+    h->busy = h->busy_ev && cudaEventRecord(h->busy_ev, h->stream) == cudaSuccess;
     if (!h->busy) cudaGetLastError();
 }
 
@@ -476,7 +475,7 @@ template <typename T>
 static cudaError_t enqueue_resident(lbm_em *h, int n, bool acc) {
     const int p = h->cur;
     return launch_resident<T>(make_args<T>(h), (const T *)h->buf[p], (T *)h->buf[1 - p], h->d_time + p,
-                              h->d_time + (1 - p), h->res, h->d_mail, h->d_ctl, n, acc, (T *)h->d_rstage,
+                              h->d_time + (1 - p), h->res, (char *)h->buf[1] + h->buf_bytes, n, acc, (T *)h->d_rstage,
                               acc ? h->ch.n_slots : 0, h->stream);
 }
 
@@ -591,8 +590,6 @@ static void free_handle(lbm_em *h) {
         dev_free(h, h->d_cs);
         dev_free(h, h->d_out);
         dev_free(h, h->d_fields);
-        dev_free(h, h->d_mail);
-        dev_free(h, h->d_ctl);
         cudaStreamSynchronize(h->stream);  // the pinned blocks are reused by other handles
     }
     if (h->g_plain) cudaGraphExecDestroy(h->g_plain);
@@ -724,9 +721,24 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
     h->buf_bytes = g->precision == LBM_EM_F16DEV ? f16_buffer_bytes(h->pstride)
                                                   : (size_t)NPLANES * h->pstride * h->elem;
     const size_t bytes = h->buf_bytes;
+    const bool always = h->prec == LBM_EM_F32 && (long long)h->nx * h->ny >= kResidentAlways;
+    if (!step_flags && !h->s4 && h->prec != LBM_EM_F16DEV && (always || h->own_stream)) {
+        TRY(h->prec == LBM_EM_F64     ? resident_plan<double>(h->nx, h->ny, h->pol, &h->res)
+            : h->prec == LBM_EM_F32X2 ? resident_plan<df>(h->nx, h->ny, h->pol, &h->res)
+                                      : resident_plan<float>(h->nx, h->ny, h->pol, &h->res),
+            "planning the resident kernel");
+        if (h->res.ctas > 0 && !always) {
+            std::lock_guard<std::mutex> lock(g_busy_mu);
+            g_sharing.push_back(h);
+            h->res_shares = true;
+        }
+    }
     for (int b = 0; b < 2; ++b) {
-        TRY(dev_alloc(h, &h->buf[b], bytes), "allocating the distributions");
-        TRY(cudaMemsetAsync(h->buf[b], 0, bytes, h->stream), "cudaMemset");
+        // (the mailboxes are cleared with the second state: an allocation and a launch of their own took
+        // 5 us of the 70 that a small handle's creation takes)
+        const size_t mail = b == 1 ? h->res.mail_bytes : 0;
+        TRY(dev_alloc(h, &h->buf[b], bytes + mail), "allocating the distributions");
+        TRY(cudaMemsetAsync(h->buf[b], 0, bytes + mail, h->stream), "cudaMemset");
     }
     TRY(dev_alloc(h, &h->d_mat, h->pstride), "allocating the material ids");
     TRY(cudaMemsetAsync(h->d_mat, 0, h->pstride, h->stream), "cudaMemset");
@@ -763,25 +775,6 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
                 "encoding the tensor maps of a state buffer");
         TRY(encode_id_map(&h->idmap, h->d_mat, h->nx, h->ny, h->pitch, kTmaTileW, kTmaTileH),
             "encoding the tensor map of the ids");
-    }
-    const bool always = h->prec == LBM_EM_F32 && (long long)h->nx * h->ny >= kResidentAlways;
-    if (!step_flags && !h->s4 && h->prec != LBM_EM_F16DEV && (always || h->own_stream)) {
-        TRY(h->prec == LBM_EM_F64     ? resident_plan<double>(h->nx, h->ny, &h->res)
-            : h->prec == LBM_EM_F32X2 ? resident_plan<df>(h->nx, h->ny, &h->res)
-                                      : resident_plan<float>(h->nx, h->ny, &h->res),
-            "planning the resident kernel");
-        if (h->res.ctas > 0) {
-            TRY(dev_alloc(h, &h->d_mail, h->res.mail_bytes), "allocating the mailboxes");
-            TRY(cudaMemsetAsync(h->d_mail, 0, h->res.mail_bytes, h->stream), "cudaMemset");
-            TRY(dev_alloc(h, &h->d_ctl, 2 * sizeof(unsigned)), "allocating the control words");
-            TRY(cudaMemsetAsync(h->d_ctl, 0, 2 * sizeof(unsigned), h->stream), "cudaMemset");
-            if (!always) {
-                TRY(cudaEventCreateWithFlags(&h->busy_ev, cudaEventDisableTiming), "cudaEventCreate");
-                std::lock_guard<std::mutex> lock(g_busy_mu);
-                g_sharing.push_back(h);
-                h->res_shares = true;
-            }
-        }
     }
     TRY(dev_alloc(h, &h->d_mtab, 256 * sizeof(MatT<double>)), "allocating the material table");
     TRY(dev_alloc(h, &h->d_time, 2 * sizeof(long long)), "allocating the time words");

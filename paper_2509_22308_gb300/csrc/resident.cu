@@ -1048,8 +1048,10 @@ int comm_warps(int warps, int rows) {
 
 }  // namespace
 
+constexpr size_t kSmemDefault = 48 * 1024;  // dynamic shared memory of a kernel that has not been given more
+
 template <typename T>
-cudaError_t resident_plan(int nx, int ny, ResidentPlan *plan) {
+cudaError_t resident_plan(int nx, int ny, int pol, ResidentPlan *plan) {
     *plan = ResidentPlan{};
     int dev = 0, sms = 0, coop = 0, smem_max = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1108,15 +1110,10 @@ cudaError_t resident_plan(int nx, int ny, ResidentPlan *plan) {
         p.mail_x = (size_t)(p.strips - 1) * ny * H * kHaloMsgs;
         mail_y = (size_t)(p.segs - 1) * 2 * H * ((nx + 1) / 2) * kHaloMsgs;
     }
-    p.mail_bytes = std::max<size_t>(2 * (p.mail_x + mail_y), 1) * sizeof(Msg);
-    for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
-        const void *f = kernel_of<T>(v & 1 ? POL_TE : POL_TM, (v & 2) != 0, p.rows);
-        int per_sm = 0;
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, (p.warps + p.comm) * 32, p.smem);
-        if (e == cudaSuccess && per_sm < 1) return cudaSuccess;
-    }
+    p.mail_bytes = kControlBytes + 2 * (p.mail_x + mail_y) * sizeof(Msg);
+    // (a block of at most the kernel's launch bounds and smem_max always fits an SM)
+    for (int acc = 0; acc < 2 && e == cudaSuccess && p.smem > kSmemDefault; ++acc)
+        e = cudaFuncSetAttribute(kernel_of<T>(pol, acc != 0, p.rows), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     p.wait = kWaitCycles;
     p.launch = p.ctas;
     if (e == cudaSuccess) *plan = p;
@@ -1125,8 +1122,8 @@ cudaError_t resident_plan(int nx, int ny, ResidentPlan *plan) {
 
 template <typename T>
 cudaError_t launch_resident(const StepArgs<T> &a, const T *fin, T *fout, const long long *t_in, long long *t_out,
-                            const ResidentPlan &plan, void *mail, unsigned *ctl, int n, bool accumulate, T *stage,
-                            int n_slots, cudaStream_t s) {
+                            const ResidentPlan &plan, void *mail, int n, bool accumulate, T *stage, int n_slots,
+                            cudaStream_t s) {
     ResidentArgs<T> r{};
     r.a = a;
     r.fin = fin;
@@ -1142,9 +1139,9 @@ cudaError_t launch_resident(const StepArgs<T> &a, const T *fin, T *fout, const l
     r.ctas = plan.ctas;
     r.n = n;
     r.wait = plan.wait;
-    r.xm = (Msg *)mail;
+    r.ctl = (unsigned *)mail;
+    r.xm = (Msg *)((char *)mail + kControlBytes);
     r.ym = r.xm + 2 * plan.mail_x;
-    r.ctl = ctl;
     r.stage = stage;
     r.n_slots = n_slots;
     void *args[] = {&r};
@@ -1159,9 +1156,9 @@ cudaError_t launch_resident(const StepArgs<T> &a, const T *fin, T *fout, const l
 }
 
 #define LBMEM_RESIDENT(T)                                                                                            \
-    template cudaError_t resident_plan<T>(int, int, ResidentPlan *);                                                 \
+    template cudaError_t resident_plan<T>(int, int, int, ResidentPlan *);                                                \
     template cudaError_t launch_resident<T>(const StepArgs<T> &, const T *, T *, const long long *, long long *,     \
-                                            const ResidentPlan &, void *, unsigned *, int, bool, T *, int, cudaStream_t);
+                                            const ResidentPlan &, void *, int, bool, T *, int, cudaStream_t);
 LBMEM_RESIDENT(float)
 LBMEM_RESIDENT(double)
 LBMEM_RESIDENT(df)

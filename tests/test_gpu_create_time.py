@@ -1,0 +1,25 @@
+"""What the plan and the mailboxes of on-chip launches add to a handle's creation: a few microseconds of about 70."""
+import time
+
+import pytest
+
+from paper_2509_22308_gb300 import lbm_em as L
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec,pol", [("f64", "tm"), ("f32", "tm"), ("f32x2", "te")])
+def test_creation_of_an_on_chip_handle(prec, pol):
+    import torch
+    kw = dict(janus=L.make_janus(8.0, 0.4, 2.0, 3.0), source=L.make_source(24), polarization=pol)
+    times = {"auto": [], "one": []}
+    for _ in range(300):
+        for mode, t in times.items():
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            s = L.Solver(64, 48, prec, steps_per_launch=mode, **kw)
+            t.append(time.perf_counter() - t0)
+            s.close()
+    auto, one = (sorted(t)[60] for t in times.values())
+    # (with two allocations and clears of their own, occupancy queries and an event: 1.2 times)
+    assert auto < 1.12 * one, (auto * 1e6, one * 1e6)
