@@ -5,6 +5,7 @@
 // distribution buffers), so a captured run of an even number of steps is replayed
 // unchanged for any start time: source phases and Fourier weights come from t.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -243,8 +244,10 @@ struct lbm_em {
     ResidentPlan res{};
     int64_t res_launches = 0;        // enqueued so far
     bool res_shares = false;         // resident only while no other such handle has steps in flight (others_busy)
-    bool busy = false;               // res_shares: busy_ev marks the end of the steps enqueued last
-    cudaEvent_t busy_ev = nullptr;
+    bool counted = false;            // in g_on_chip
+    bool watched = false;            // in g_watched: marks its steps in flight
+    bool busy = false;               // busy_ev marks the end of the steps enqueued last
+    cudaEvent_t busy_ev = nullptr;   // created with the first mark
     int tma3_ctas = 0;
     int tma_ctas = 0;
     // contour and accumulators
@@ -440,26 +443,41 @@ static lbm_em_status build_graph(lbm_em *h, bool acc, cudaGraphExec_t *out) {
 // time on streams of their own fill it together (7 handles, GLUPS with plain / resident launches:
 // FP32 128^2 38 / 22, 256^2 97 / 65, 320^2 99 / 96, 400^2 94 / 132, 512^2 107 / 142; FP64 128^2
 // 15 / 12, 256^2 18.2 / 16.5, 512^2 18.5 / 17.8; double-float 256^2 42 / 18).  So FP32 lattices of at
-// least kResidentAlways sites always take resident launches, the others only on the library's own
-// stream and while no other handle of that kind has steps in flight; a caller's stream keeps its
-// plain launches.  The bits are the same either way.
-static const long long kResidentAlways = 330 * 330;
+// least kResidentAlways sites take resident launches beside others of the on-chip kind, the rest of
+// that kind only on the library's own stream and while no other of them has steps in flight; a caller's
+// stream keeps its plain launches.  The bits are the same either way.
+//
+// Beside a handle that has plain launches in flight on another stream, an on-chip handle takes plain ones
+// too if that one leaves it room (ms for 1920 steps of each, plain / resident: FP32 512^2 + FP16-deviation
+// 512^2 10.6 / 12.2; FP32 350^2 + FP32 512^2 with the two-step flag 8.3 / 9.8; FP64 256^2 + FP64 600^2 48.5 /
+// 53.2; double-float 200^2 + 512^2 17.0 / 21.4).  The four-step kernel does not (FP64 256^2 + FP32 800^2 23.5 /
+// 19.2, + FP32 2048^2 36.2 / 30.0), nor do other launches from kAloneSites sites on (+ FP64 1024^2 73.7 /
+// 70.0), nor, beside FP64, whose plain launches are twice as slow, ones with a state below kSmallState
+// (FP64 256^2 + FP16-deviation 512^2 17.8 / 15.8, 128^2 + 256^2 10.1 / 6.1).
+static const long long kResidentAlways = 330 * 330, kAloneSites = 1LL << 20;
+static const size_t kSmallState = 16 << 20;
+// Calls of fewer steps are not marked as in flight by handles with plain launches (the record takes
+// about 1 us), nor any while no on-chip handle exists.
+static const int kMarkSteps = 16;
 static std::mutex g_busy_mu;
-static std::vector<lbm_em *> g_sharing;  // the live handles with res_shares
+static std::vector<lbm_em *> g_watched;   // the live handles that mark their steps in flight
+static std::atomic<int> g_on_chip{0};     // live handles with a resident plan
 
+// Whether handles that h should not displace have steps in flight on other streams.
 static bool others_busy(const lbm_em *h) {
     std::lock_guard<std::mutex> lock(g_busy_mu);
-    // the query is legal whatever other threads capture
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
     bool busy = false;
-    for (lbm_em *o : g_sharing)
-        if (o != h && o->dev == h->dev && o->busy) {
-            o->busy = cudaEventQuery(o->busy_ev) == cudaErrorNotReady;
-            busy = busy || o->busy;
-        }
-    cudaGetLastError();
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    for (lbm_em *o : g_watched) {
+        if (!o->busy || o->dev != h->dev || o->stream == h->stream) continue;
+        if (o->res_shares ? !h->res_shares : h->prec == LBM_EM_F64 && o->buf_bytes < kSmallState) continue;
+        // the query is legal whatever other threads capture
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        o->busy = cudaEventQuery(o->busy_ev) == cudaErrorNotReady;
+        cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        busy = busy || o->busy;
+    }
     return busy;
 }
 
@@ -468,6 +486,19 @@ static void mark_busy(lbm_em *h) {
     if (!h->busy_ev && cudaEventCreateWithFlags(&h->busy_ev, cudaEventDisableTiming) != cudaSuccess) h->busy_ev = nullptr;
     h->busy = h->busy_ev && cudaEventRecord(h->busy_ev, h->stream) == cudaSuccess;
     if (!h->busy) cudaGetLastError();
+}
+
+static void watch(lbm_em *h) {
+    std::lock_guard<std::mutex> lock(g_busy_mu);
+    g_watched.push_back(h);
+    h->watched = true;
+}
+
+static void unwatch(lbm_em *h) {
+    if (h->counted) --g_on_chip;
+    if (!h->watched) return;
+    std::lock_guard<std::mutex> lock(g_busy_mu);
+    g_watched.erase(std::remove(g_watched.begin(), g_watched.end(), h), g_watched.end());
 }
 
 // n steps (at most kResidentSteps, accumulating kResidentAccSteps) in one resident launch.
@@ -503,7 +534,10 @@ static bool stream_capturing(const lbm_em *h) {
 static lbm_em_status run_steps(lbm_em *h, int64_t n, bool acc) {
     const int m = launch_steps(h, acc), gs = graph_steps(h, acc);
     const bool capable = h->res.ctas > 0 && n >= kResidentMin && !stream_capturing(h);
-    if (capable && !(h->res_shares && others_busy(h))) {
+    const bool marks = h->watched && (h->res_shares ? capable
+                                                    : n >= kMarkSteps && g_on_chip.load(std::memory_order_relaxed) > 0 &&
+                                                          !stream_capturing(h));
+    if (capable && !others_busy(h)) {
         const int64_t most = acc ? kResidentAccSteps : kResidentSteps;
         while (n > 0) {
             const int c = (int)(n / ((n + most - 1) / most));  // launches of about the same length
@@ -554,7 +588,7 @@ static lbm_em_status run_steps(lbm_em *h, int64_t n, bool acc) {
             n -= 1;
         }
     }
-    if (capable && h->res_shares) mark_busy(h);
+    if (marks) mark_busy(h);
     return LBM_EM_OK;
 }
 
@@ -574,10 +608,7 @@ static void free_contour(lbm_em *h) {
 
 static void free_handle(lbm_em *h) {
     if (!h) return;
-    if (h->res_shares) {
-        std::lock_guard<std::mutex> lock(g_busy_mu);
-        g_sharing.erase(std::remove(g_sharing.begin(), g_sharing.end(), h), g_sharing.end());
-    }
+    unwatch(h);
     cudaSetDevice(h->dev);
     if (h->stream) {
         free_contour(h);
@@ -727,12 +758,11 @@ static lbm_em_status create_common(const lbm_em_grid *g, const lbm_em_source *s,
             : h->prec == LBM_EM_F32X2 ? resident_plan<df>(h->nx, h->ny, h->pol, &h->res)
                                       : resident_plan<float>(h->nx, h->ny, h->pol, &h->res),
             "planning the resident kernel");
-        if (h->res.ctas > 0 && !always) {
-            std::lock_guard<std::mutex> lock(g_busy_mu);
-            g_sharing.push_back(h);
-            h->res_shares = true;
-        }
     }
+    h->counted = h->res.ctas > 0;
+    h->res_shares = h->counted && !always;
+    if (h->counted) ++g_on_chip;
+    if (h->res_shares || (!h->counted && !h->s4 && (long long)h->nx * h->ny < kAloneSites)) watch(h);
     for (int b = 0; b < 2; ++b) {
         // (the mailboxes are cleared with the second state: an allocation and a launch of their own took
         // 5 us of the 70 that a small handle's creation takes)

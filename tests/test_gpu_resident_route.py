@@ -93,3 +93,38 @@ def test_a_captured_stream_and_steps_in_flight_elsewhere_take_plain_launches():
         b.step(50)
         b.sync()
         assert b.resident_launches() == 2
+
+
+# the handle that is in flight, the on-chip one beside it, and whether that takes on-chip launches meanwhile
+@pytest.mark.parametrize("first,second,resident", [
+    (("f16dev", 512, "auto"), ("f32", 512), False), (("f32", 512, "two"), ("f32", 350), False), (("f32", 512, "two"), ("f32", 128), False),
+    (("f64", 600, "auto"), ("f64", 256), False), (("f32x2", 512, "auto"), ("f32x2", 200), False),
+    (("f32", 400, "auto"), ("f32", 512), True),     # both on chip and of the size that always is
+    (("f32", 2048, "auto"), ("f64", 128), True), (("f32", 800, "auto"), ("f64", 256), True),  # four steps per launch
+    (("f64", 1100, "auto"), ("f32", 400), True),    # fills the GPU by itself
+    (("f16dev", 256, "auto"), ("f64", 128), True)])  # little in the way of FP64
+@pytest.mark.parametrize("streams", ["own", "caller's", "one"])
+def test_steps_in_flight_of_other_kinds(first, second, resident, streams):
+    import torch
+    (prec_a, na, spl), (prec_b, nb) = first, second
+    if streams != "own" and not (prec_b == "f32" and nb >= 330):
+        pytest.skip("plain on a caller's stream")
+    st = {"own": [None, None], "caller's": [torch.cuda.Stream(), torch.cuda.Stream()], "one": [torch.cuda.Stream()] * 2}[streams]
+    j, src = L.make_janus(20.0, 0.4, 2.0, 3.0), L.make_source(24)
+    with L.Solver(na, na, prec_a, janus=j, source=src, stream=st[0], steps_per_launch=spl) as a, \
+            L.Solver(nb, nb, prec_b, janus=j, source=src, stream=st[1]) as b, \
+            L.Solver(nb, nb, prec_b, janus=j, source=src, stream=st[1], steps_per_launch="one") as ref:
+        b.step(48)
+        b.sync()
+        n = b.resident_launches()
+        assert n == 1
+        a.step(9600)  # tens of milliseconds
+        b.step(48)
+        ref.step(96)
+        assert b.resident_launches() - n == int(resident or streams == "one")  # (one stream: nothing runs beside it)
+        a.sync()
+        b.step(48)
+        ref.step(48)
+        assert b.resident_launches() - n == 1 + int(resident or streams == "one")
+        for u, v in zip(b.fields(), ref.fields()):
+            assert np.array_equal(u, v)
