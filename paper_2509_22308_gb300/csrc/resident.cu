@@ -40,17 +40,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// What one lane holds of a row: two adjacent sites in FP32, one site in the 8-byte forms.
-template <typename T>
-struct Form {
-    using V = T;
-    static constexpr int CPL = 1, MSGS = 2;  // 16-byte messages per border site
-};
-template <>
-struct Form<float> {
-    using V = f2;
-    static constexpr int CPL = 2, MSGS = 1;
-};
+constexpr int MSGS = 2;  // 8-byte forms: 16-byte messages per border site
 
 __device__ __forceinline__ df shfl_from(df v, int d) {  // d = -1: the lane to the left, +1: to the right
     const int src = ((int)threadIdx.x & 31) + d;
@@ -74,7 +64,7 @@ __device__ __forceinline__ T from_right(T v, T in, int lane) {
 }
 // The lattice's last column keeps its own value (zero-gradient open edge).
 template <typename T>
-__device__ __forceinline__ T keep_last(T pulled, T own, bool a_last, bool) { return a_last ? own : pulled; }
+__device__ __forceinline__ T keep_last(T pulled, T own, bool a_last) { return a_last ? own : pulled; }
 __device__ __forceinline__ f2 keep_last(f2 pulled, f2 own, bool a_last, bool b_last) {
     return pack2(a_last ? lo2(own) : lo2(pulled), b_last ? hi2(own) : hi2(pulled));
 }
@@ -100,9 +90,12 @@ __device__ __forceinline__ void store_cols(float *p, int xa, int nx, f2 v) {
 }
 
 // ---- messages -----------------------------------------------------------------------------
-// One 16-byte access each way.  Every word of a message is looked at by its receiver: where a word was
-// not, the compiler narrowed the 128-bit load to two smaller ones, between which a message can arrive
-// (seen as a value of the message before under the new sequence number).
+// One 16-byte access each way.  Every word of a message has to be looked at by its receiver: where a word
+// was not, the compiler narrowed the 128-bit load to two smaller ones, between which a message can arrive
+// (seen as a value of the message before under the new sequence number).  So whoever takes a message apart
+// (from_word, take_pair) uses all of its values, and all_there, get_row, get_site and watch_mail
+// compare all of its sequence numbers: a value that is no longer needed must leave the message, not just
+// go unused.
 struct alignas(16) Msg {
     unsigned long long v, seq;
 };
@@ -121,6 +114,7 @@ __device__ __forceinline__ void msg_store(Msg *p, unsigned long long v, unsigned
 }
 __device__ __forceinline__ unsigned long long word_of(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ unsigned long long word_of(df v) { return pack2(v.hi, v.lo).v; }
+// (both words of a message are used: see Msg)
 __device__ __forceinline__ void from_word(unsigned long long w, double &v) { v = __longlong_as_double((long long)w); }
 __device__ __forceinline__ void from_word(unsigned long long w, df &v) { v = df(lo2(f2{w}), hi2(f2{w})); }
 
@@ -234,10 +228,10 @@ __host__ __device__ inline ResidentSmem resident_smem(int warps, int rows) {
     o.src = o.table + 256 * sizeof(MatT<T>);
     o.flags = o.src + (size_t)kResidentSteps * 2 * sizeof(T);
     o.xin = o.flags + 2 * kResidentMaxWarps * sizeof(unsigned);
-    o.yin = o.xin + (size_t)2 * warps * rows * 2 * Form<T>::MSGS * sizeof(Msg);
+    o.yin = o.xin + (size_t)2 * warps * rows * 2 * MSGS * sizeof(Msg);
     o.ids = o.yin + (size_t)2 * 128 * sizeof(Msg);
-    o.slots = o.ids + ((size_t)warps * rows * 32 * Form<T>::CPL + 15) / 16 * 16;
-    o.end = o.slots + (size_t)warps * rows * 32 * Form<T>::CPL * sizeof(int);
+    o.slots = o.ids + ((size_t)warps * rows * 32 + 15) / 16 * 16;
+    o.end = o.slots + (size_t)warps * rows * 32 * sizeof(int);
     return o;
 }
 
@@ -285,7 +279,6 @@ constexpr int kWatch = 4;
 template <typename T>
 __device__ void watch_mail(const ResidentArgs<T> &r, unsigned base, int cw, int lane, Msg *xin, int xin_slot,
                            Msg *y_above, Msg *y_below, int yin_slot) {
-    constexpr int MSGS = Form<T>::MSGS;
     const int ny = r.a.ny, first = (int)blockIdx.x * r.warps, warps = min(r.warps, r.total - first);
     const int n_x = warps * r.rows * 2 * MSGS;
     const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * MSGS, yslot = (size_t)r.ctas * 2 * 64;
@@ -450,6 +443,7 @@ __device__ __forceinline__ bool all_there(const Msg *m, unsigned seq) {
     for (int i = 0; i < kHaloMsgs; ++i) ok = ok && (unsigned)(m[i].seq >> 32) == seq;
     return ok && (unsigned)(m[kHaloMsgs - 1].v >> 32) == seq && (unsigned)m[kHaloMsgs - 1].seq == seq;
 }
+// (every value of the messages is used: see Msg)
 __device__ __forceinline__ void take_pair(const Msg *m, Pop<f2> &s) {
     float v[24];
 #pragma unroll
@@ -675,9 +669,7 @@ __global__ void __launch_bounds__(resident32_warps(R) * 32, 1)
 // 11.7 us.
 template <typename T, int POL, bool ACC>
 __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __grid_constant__ ResidentArgs<T> r) {
-    using F = Form<T>;
-    using V = typename F::V;
-    constexpr int CPL = F::CPL, W = 32 * CPL;
+    constexpr int W = 32;
     extern __shared__ __align__(16) unsigned char sm[];
     const StepArgs<T> &a = r.a;
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
@@ -688,8 +680,8 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     const int loc = warp < r.warps ? quarter * per + min(quarter, extra) + (warp >> 2) : warp;
     const int nx = a.nx, ny = a.ny;
     const ResidentSmem o = resident_smem<T>(r.warps, r.rows);
-    V *const st = reinterpret_cast<V *>(sm) + (size_t)loc * r.rows * NPLANES * 32 + lane;
-    V *const edge = reinterpret_cast<V *>(sm + o.edge);
+    T *const st = reinterpret_cast<T *>(sm) + (size_t)loc * r.rows * NPLANES * 32 + lane;
+    T *const edge = reinterpret_cast<T *>(sm + o.edge);
     MatT<T> *const table = reinterpret_cast<MatT<T> *>(sm + o.table);
     T *const srcv = reinterpret_cast<T *>(sm + o.src);
     unsigned *const flags = reinterpret_cast<unsigned *>(sm + o.flags);
@@ -704,13 +696,12 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     const int g = (int)blockIdx.x * r.warps + loc;
     const bool live = warp < r.warps && g < r.total;  // a compute warp with rows
     const int strip = live ? g / r.segs : 0, seg = live ? g - strip * r.segs : 0;
-    const int x0 = strip * W, xa = x0 + lane * CPL;
+    const int x0 = strip * W, xa = x0 + lane;
     const int y0 = (int)((long long)seg * ny / r.segs);
     const int nrows = live ? (int)((long long)(seg + 1) * ny / r.segs) - y0 : 0;
     const bool has_left = strip > 0, has_right = strip + 1 < r.strips, has_up = seg > 0, has_down = seg + 1 < r.segs;
     const bool up_here = has_up && loc > 0, down_here = has_down && loc + 1 < r.warps;  // neighbour in this block
-    const bool a_last = xa == nx - 1, b_last = CPL == 2 && xa + 1 == nx - 1;
-    const bool in_a = xa < nx, in_b = xa + CPL - 1 < nx;
+    const bool last_column = xa == nx - 1, inside = xa < nx;
     const int kind = a.src.kind;
     const size_t ps = a.pstride;
 
@@ -724,18 +715,13 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         const size_t row = (size_t)(y0 + i) * a.pitch;
 #pragma unroll
         for (int p = 0; p < NPLANES; ++p) st[(i * NPLANES + p) * 32] = load_cols(r.fin + p * ps + row, xa, nx);
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) {
-            const bool in = xa + c < nx;
-            const uint8_t id = in ? a.mat[row + xa + c] : (uint8_t)0;
-            ids[i * W + lane * CPL + c] = id;
-            if (ACC)
-                slots[i * W + lane * CPL + c] =
-                    in && y0 + i >= a.accp.y0 && y0 + i <= a.accp.y1 ? a.accp.slot[row + xa + c] : -1;
-            if (in) {
-                if (id0 < 0) id0 = id;
-                uniform = uniform && id == id0;
-            }
+        const uint8_t id = inside ? a.mat[row + xa] : (uint8_t)0;
+        ids[i * W + lane] = id;
+        if (ACC)
+            slots[i * W + lane] = inside && y0 + i >= a.accp.y0 && y0 + i <= a.accp.y1 ? a.accp.slot[row + xa] : -1;
+        if (inside) {
+            if (id0 < 0) id0 = id;
+            uniform = uniform && id == id0;
         }
     }
     // one material over all of the warp's sites: its constants stay in registers
@@ -749,10 +735,10 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     // mailboxes: xm[slot][strip border][0: going right, 1: going left][row][message],
     // ym[slot][receiving block][0: from above, 1: from below][message][lane]; inboxes:
     // xin[slot][warp][row][0: from the left, 1: from the right][message], yin[slot][0, 1][message][lane]
-    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * F::MSGS, yslot = (size_t)r.ctas * 2 * 64;
-    const int xin_slot = r.warps * r.rows * 2 * F::MSGS;
+    const size_t xslot = (size_t)max(r.strips - 1, 0) * 2 * ny * MSGS, yslot = (size_t)r.ctas * 2 * 64;
+    const int xin_slot = r.warps * r.rows * 2 * MSGS;
     Msg *const xin = reinterpret_cast<Msg *>(sm + o.xin), *const yin = reinterpret_cast<Msg *>(sm + o.yin);
-    Msg *const my_xin = xin + loc * r.rows * 2 * F::MSGS;
+    Msg *const my_xin = xin + loc * r.rows * 2 * MSGS;
     const size_t bstep = (size_t)r.warps * 128;
     // nothing has arrived yet for the second step (shared memory holds what an earlier kernel left,
     // perhaps a message of this very number)
@@ -764,7 +750,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         if (mine)
             for (int i = 0; i < nrows; ++i) {
                 const size_t at = (size_t)(y0 + i) * a.pitch + (lane == 0 ? x0 - 1 : x0 + W);
-                put_site(my_xin + (base & 1u) * xin_slot + (i * 2 + (lane == 0 ? 0 : 1)) * F::MSGS,
+                put_site(my_xin + (base & 1u) * xin_slot + (i * 2 + (lane == 0 ? 0 : 1)) * MSGS,
                             r.fin[(lane == 0 ? P_EPX : P_EMX) * ps + at], r.fin[(lane == 0 ? P_HXPX : P_HXMX) * ps + at],
                             base);
             }
@@ -778,16 +764,16 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
             put_row(yin + (base & 1u) * 128 + 64 + lane, load_cols(r.fin + P_EMY * ps + row, xa, nx),
                     load_cols(r.fin + P_HYMY * ps + row, xa, nx), base);
         }
-        V *const e = edge + bstep + loc * 128 + lane;
-        const V *const ql = st + (nrows - 1) * NPLANES * 32;
+        T *const e = edge + bstep + loc * 128 + lane;
+        const T *const ql = st + (nrows - 1) * NPLANES * 32;
         e[0] = st[P_EMY * 32], e[32] = st[P_HYMY * 32], e[64] = ql[P_EPY * 32], e[96] = ql[P_HYPY * 32];
     }
-    Msg *const x_send = r.xm + (((size_t)(lane == 0 ? strip - 1 : strip) * 2 + (lane == 0 ? 1 : 0)) * ny + y0) * F::MSGS;
+    Msg *const x_send = r.xm + (((size_t)(lane == 0 ? strip - 1 : strip) * 2 + (lane == 0 ? 1 : 0)) * ny + y0) * MSGS;
     const bool sends_x = (lane == 0 && has_left) || (lane == 31 && has_right);
     Msg *const up_send = r.ym + ((size_t)blockIdx.x - 1) * 128 + 64 + lane;
     Msg *const down_send = r.ym + ((size_t)blockIdx.x + 1) * 128 + lane;
-    const RowLink<V> up{has_up, up_here, flags + 2 * (loc - 1) + 1, edge + ((loc - 1) * 4 + 2) * 32 + lane, yin + lane};
-    const RowLink<V> dn{has_down, down_here, flags + 2 * (loc + 1), edge + ((loc + 1) * 4) * 32 + lane,
+    const RowLink<T> up{has_up, up_here, flags + 2 * (loc - 1) + 1, edge + ((loc - 1) * 4 + 2) * 32 + lane, yin + lane};
+    const RowLink<T> dn{has_down, down_here, flags + 2 * (loc + 1), edge + ((loc + 1) * 4) * 32 + lane,
                         yin + 64 + lane};
     __syncthreads();  // the only block barrier: from here on a warp waits for its neighbours alone
 
@@ -803,13 +789,13 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
     const bool waits_x = lane == 0 ? has_left : lane == 31 && has_right;
 
     // The border row of step k - 1 from a neighbouring segment; false: gave up.
-    auto receive = [&](const RowLink<V> &l, int k, V &v, V &h) -> bool {
+    auto receive = [&](const RowLink<T> &l, int k, T &v, T &h) -> bool {
         Patience pt;
         if (l.here) {
             // by a vote, like every wait here: over() needs all lanes, and each lane's own acquire orders its reads
             while (!__all_sync(kFull, (int)(flag_get(l.flag) - (unsigned)k) >= 0))
                 if (pt.over(r)) return false;
-            const V *const q = l.buf + ((k + 1) & 1) * bstep;
+            const T *const q = l.buf + ((k + 1) & 1) * bstep;
             v = q[0];
             h = q[32];
             return true;
@@ -830,20 +816,20 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
         const int PC0 = DOWN ? P_EPY : P_EMY, PC1 = DOWN ? P_HYPY : P_HYMY;
         const int PN0 = DOWN ? P_EMY : P_EPY, PN1 = DOWN ? P_HYMY : P_HYPY;
         const int RS = (DOWN ? 1 : -1) * NPLANES * 32;
-        const RowLink<V> &la = DOWN ? up : dn, &lb = DOWN ? dn : up;
+        const RowLink<T> &la = DOWN ? up : dn, &lb = DOWN ? dn : up;
         const int ifirst = DOWN ? 0 : nrows - 1;
         for (int k = 0; k < r.n; ++k) {
             const unsigned seq = base + (unsigned)k, so = seq + 1u;
             const bool sends = k + 1 < r.n;
             const bool src_now = strip == 0 && kind != SRC_NONE && t0 + k >= 1, inner = has_left || has_right;
-            V *q = st + ifirst * NPLANES * 32;
+            T *q = st + ifirst * NPLANES * 32;
             // beyond the lattice's top and bottom: the border row's own values (zero-gradient open edge)
-            V c0 = q[PC0 * 32], c1 = q[PC1 * 32];
+            T c0 = q[PC0 * 32], c1 = q[PC1 * 32];
             if (la.exists && !receive(la, k, c0, c1)) return false;
-            V *const eout = edge + (k & 1) * bstep + loc * 128 + lane;
+            T *const eout = edge + (k & 1) * bstep + loc * 128 + lane;
             Msg *const xs = x_send + (so & 1u) * xslot;
             // the pair that row i (at w) pulls from the row taken after it; false: gave up
-            auto next = [&](const V *w, bool last, V &n0, V &n1) -> bool {
+            auto next = [&](const T *w, bool last, T &n0, T &n1) -> bool {
                 if (!last) {
                     n0 = w[RS + PN0 * 32], n1 = w[RS + PN1 * 32];
                     return true;
@@ -852,16 +838,16 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                 return !lb.exists || receive(lb, k, n0, n1);
             };
             // row i (at w) pulled from its neighbours, and its own pair carried to the row taken after it
-            auto pull = [&](const V *w, int i, V n0, V n1, Pop<V> &p) -> bool {
+            auto pull = [&](const T *w, int i, T n0, T n1, Pop<T> &p) -> bool {
                 // the border values from the left (lane 0) and the right (lane 31)
                 T in0{}, in1{};
                 if (inner) {
-                    const Msg *const xr = my_xin + (seq & 1u) * xin_slot + (i * 2 + (lane == 0 ? 0 : 1)) * F::MSGS;
+                    const Msg *const xr = my_xin + (seq & 1u) * xin_slot + (i * 2 + (lane == 0 ? 0 : 1)) * MSGS;
                     Patience pt;
                     while (!__all_sync(kFull, !waits_x || get_site<T>(xr, in0, in1, seq)))
                         if (pt.over(r)) return false;
                 }
-                const V epx = w[P_EPX * 32], emx = w[P_EMX * 32], hxpx = w[P_HXPX * 32], hxmx = w[P_HXMX * 32];
+                const T epx = w[P_EPX * 32], emx = w[P_EMX * 32], hxpx = w[P_HXPX * 32], hxmx = w[P_HXMX * 32];
                 p.ez = w[P_EZ * 32];
                 p.hxz = w[P_HXZ * 32];
                 p.hyz = w[P_HYZ * 32];
@@ -877,14 +863,14 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                 p.emx = from_right(emx, in0, lane);
                 p.hxmx = from_right(hxmx, in1, lane);
                 if (!has_right) {
-                    p.emx = keep_last(p.emx, emx, a_last, b_last);
-                    p.hxmx = keep_last(p.hxmx, hxmx, a_last, b_last);
+                    p.emx = keep_last(p.emx, emx, last_column);
+                    p.hxmx = keep_last(p.hxmx, hxmx, last_column);
                 }
                 if (src_now && lane == 0) inject_source_t<T>(kind, srcv[2 * k], srcv[2 * k + 1], p);
                 return true;
             };
             // the updated row i (to w): its fields staged, its populations kept and sent
-            auto put = [&](V *w, int i, const Pop<V> &p, const T *f3) {
+            auto put = [&](T *w, int i, const Pop<T> &p, const T *f3) {
                 if constexpr (ACC) {
                     const int y = y0 + i;
                     if (y >= a.accp.y0 && y <= a.accp.y1) {
@@ -930,8 +916,8 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                 }
             };
             for (int j = 0, i = ifirst; j < nrows; ++j, i += DOWN ? 1 : -1, q += RS) {
-                V n0, n1;
-                Pop<V> p;
+                T n0, n1;
+                Pop<T> p;
                 T f3[3];
                 if constexpr (std::is_same<T, df>::value) {
                     // two rows at a time as packed pairs (an odd last one with itself).  The first is sent no
@@ -940,14 +926,14 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                     const bool pair = j + 1 < nrows;
                     const int i2 = pair ? i + (DOWN ? 1 : -1) : i;
                     if (!next(q, !pair, n0, n1) || !pull(q, i, n0, n1, p)) return false;
-                    Pop<V> p2 = p;
+                    Pop<T> p2 = p;
                     if (pair && (!next(q + RS, j + 2 == nrows, n0, n1) || !pull(q + RS, i2, n0, n1, p2))) return false;
                     Pop<df2> v;
                     df2 g3[3];
                     each_of_pair(v, p, p2, [](df2 &o, df &u, df &w) { o = pack_df(u, w); });
                     rw |= update_pair<POL, ACC>(v, uniform ? mu : table[ids[i * 32 + lane]],
                                                 uniform ? mu : table[ids[i2 * 32 + lane]], true, a.runaway, g3) &&
-                          in_a;
+                          inside;
                     each_of_pair(v, p, p2, [](df2 &o, df &u, df &w) { u = first(o), w = second(o); });
                     if (ACC) f3[0] = first(g3[0]), f3[1] = first(g3[1]), f3[2] = first(g3[2]);
                     put(q, i, p, f3);
@@ -957,7 +943,7 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1) k_resident(const __
                     ++j, i = i2, q += RS;
                 } else {
                     if (!next(q, j + 1 == nrows, n0, n1) || !pull(q, i, n0, n1, p)) return false;
-                    update_row<POL, ACC>(p, uniform ? mu : table[ids[i * 32 + lane]], a.runaway, in_a, rw, f3);
+                    update_row<POL, ACC>(p, uniform ? mu : table[ids[i * 32 + lane]], a.runaway, inside, rw, f3);
                     put(q, i, p, f3);
                 }
             }
@@ -1041,9 +1027,8 @@ const void *kernel_of(int pol, bool acc, int rows) {
 }
 
 // Communication warps for `warps` compute warps of `rows` rows.
-template <typename T>
 int comm_warps(int warps, int rows) {
-    return (warps * rows * 2 * Form<T>::MSGS + 128 + 32 * kWatch - 1) / (32 * kWatch);
+    return (warps * rows * 2 * MSGS + 128 + 32 * kWatch - 1) / (32 * kWatch);
 }
 
 }  // namespace
@@ -1060,9 +1045,6 @@ cudaError_t resident_plan(int nx, int ny, int pol, ResidentPlan *plan) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess || !coop) return e;
     ResidentPlan p{};
-    const int W = 32 * Form<T>::CPL;
-    p.strips = (nx + W - 1) / W;
-    const long long units = (long long)p.strips * ny;  // rows of strips
     bool fits = false;
     if (std::is_same<T, float>::value) {
         p.strips = nx <= 64 ? 1 : (nx - 2 * H + 63 - 2 * H) / (64 - 2 * H);
@@ -1087,12 +1069,14 @@ cudaError_t resident_plan(int nx, int ny, int pol, ResidentPlan *plan) {
         p.total = p.strips * p.segs * p.warps;
     } else {
         // as many warps per block as there are rows of strips per SM, fewer where they do not fit
+        p.strips = (nx + 31) / 32;
+        const long long units = (long long)p.strips * ny;  // rows of strips
         for (p.warps = (int)std::min<long long>((units + sms - 1) / sms, kResidentMaxWarps - 1); p.warps >= 1 && !fits; --p.warps) {
             p.segs = std::min((int)((long long)sms * p.warps / p.strips), ny);
             if (p.segs < 1) break;
             p.rows = (ny + p.segs - 1) / p.segs;
             p.total = p.strips * p.segs;
-            p.comm = comm_warps<T>(p.warps, p.rows);
+            p.comm = comm_warps(p.warps, p.rows);
             p.smem = resident_smem<T>(p.warps, p.rows).end;
             fits = p.warps + p.comm <= kResidentMaxWarps && p.rows <= kResidentMaxRows && p.smem <= (size_t)smem_max;
             if (fits) break;
@@ -1104,7 +1088,7 @@ cudaError_t resident_plan(int nx, int ny, int pol, ResidentPlan *plan) {
     }
     if (!fits) return cudaSuccess;
     p.ctas = (p.total + p.warps - 1) / p.warps;
-    p.mail_x = (size_t)(p.strips - 1) * 2 * ny * Form<T>::MSGS;
+    p.mail_x = (size_t)(p.strips - 1) * 2 * ny * MSGS;
     size_t mail_y = (size_t)p.ctas * 2 * 64;
     if (std::is_same<T, float>::value) {
         p.mail_x = (size_t)(p.strips - 1) * ny * H * kHaloMsgs;

@@ -63,7 +63,7 @@ static_assert(LW == 64 && OUTW + 2 * HALO == LW && HALO % 4 == 0 && HALO >= BT,
               "two sites per lane, a 16-byte aligned halo as wide as the steps");
 static_assert(IDBOX >= LW + 12 && IDBOX % 16 == 0, "the id box covers the strip from any 16-byte boundary");
 
-// Shared memory: the material table, then per warp RING row slots (state row, id row) and the
+// Shared memory: the material table (of a single lattice; a batch's warps have their own), then per warp RING row slots (state row, id row) and the
 // -y pairs of the last lattice row per level (the bottom edge, see below).  Level 0 (the stored
 // state) is read straight from the slots, so a row's slot stays in use until the row two further
 // on has arrived: 5 slots, 3 rows in use and 2 in flight.  The FP16-deviation form's copies
@@ -81,7 +81,8 @@ struct Layout {
     static constexpr size_t EDGE = BT * 32 * sizeof(float4);
     static constexpr size_t WARP = RING * SLOT + EDGE;
     static constexpr size_t TABLE = 256 * sizeof(MatT<float>);
-    static constexpr size_t SMEM = TABLE + NW * WARP + 128;  // + alignment slack
+    static constexpr size_t BATCH_SMEM = NW * WARP + 128;  // + alignment slack
+    static constexpr size_t SMEM = TABLE + BATCH_SMEM;
 };
 static_assert(3 * (Layout<false>::SMEM + 1024 + 256) <= 233472 && 3 * (Layout<true>::SMEM + 1024 + 256) <= 233472,
               "three blocks per SM");
@@ -256,7 +257,7 @@ __device__ __forceinline__ void take_row(unsigned char *sl, int lane, float inv_
 struct UnitCtx {
     int nx, ny, pitch, kind;
     unsigned runaway;
-    int ay0, ay1, period;
+    int ay0, ay1;
     size_t pstride;
     float scale, inv_scale;                       // FP16-deviation form
     unsigned short nis;                           // -inv_scale in FP16 (the MIX kernel)
@@ -265,8 +266,6 @@ struct UnitCtx {
     float *fe_out, *fhx_out, *fhy_out;
     long long acc_from, steps;
     const int *slot;                              // the lattice's slot map (pitch layout)
-    double *acc;                                  // its accumulators (6 per slot)
-    const double2 *cs;                            // (cos w t, sin w t) for t mod period
     float *stage;                                 // ACC: 12 staged FP32 fields per slot (see stream_unit)
 };
 
@@ -719,7 +718,7 @@ __global__ void __launch_bounds__(NW * 32, 3)
     __shared__ SrcLevels sp[NW];         // its source values (first strip), per warp
     unsigned char *s = sm_dyn + ((128u - (smem_u32(sm_dyn) & 127u)) & 127u);
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    unsigned char *ring = s + LY::TABLE + (size_t)warp * LY::WARP;
+    unsigned char *ring = s + (size_t)warp * LY::WARP;
     const long long t = *t_in;
     if (blockIdx.x == 0 && threadIdx.x == 0) *t_out = t + BT;
     if (lane == 0) {
@@ -746,14 +745,12 @@ __global__ void __launch_bounds__(NW * 32, 3)
             u.runaway = I.runaway;
             u.ay0 = I.ay0;
             u.ay1 = I.ay1;
-            u.period = I.period;
             u.pstride = (size_t)I.pstride;
             u.fout = buf_out + I.base;
             u.acc_from = I.acc_from;
             u.steps = steps;
             u.slot = slot + I.slot_base;
             u.stage = stage + 12 * (size_t)I.acc_base;
-            u.cs = I.cs;
         }
         UnitRun &r = urun[warp];
         if (lane == 0) {
@@ -944,7 +941,7 @@ cudaError_t encode_stream_maps(CUtensorMap *smap, CUtensorMap *fmap, CUtensorMap
 template <int POL, bool ACC>
 cudaError_t allow_smem_batch4() {
     return cudaFuncSetAttribute(k_batch_step4<POL, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Layout<false>::SMEM);
+                                (int)Layout<false>::BATCH_SMEM);
 }
 
 cudaError_t batch_stream_prepare(int *resident_warps) {
@@ -957,7 +954,7 @@ cudaError_t batch_stream_prepare(int *resident_warps) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step4<POL_TM, false>, NW * 32,
-                                                          Layout<false>::SMEM);
+                                                          Layout<false>::BATCH_SMEM);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     if (e == cudaSuccess) *resident_warps = per_sm * sms * NW;
     return e;
@@ -974,7 +971,7 @@ cudaError_t launch_batch_step4(const StreamInst *insts, const SourceParams *srcp
                                const int *n_units, const CUtensorMap *maps, int p, float *buf_out, const int *slot, double *acc,
                                float *stage, const int *slot_inst, int n_slots, unsigned *err, const long long *t_in,
                                long long *t_out, int grid, int pol, bool accumulate, cudaStream_t s) {
-    const size_t sm = Layout<false>::SMEM;
+    const size_t sm = Layout<false>::BATCH_SMEM;
     auto run = [&](auto kernel) {
         kernel<<<grid, NW * 32, sm, s>>>(insts, units, n_units, srcp, maps, p, buf_out, slot, stage, err, t_in, t_out);
     };
@@ -1019,9 +1016,6 @@ cudaError_t launch_step4_stream(const StepArgs<float> &sa, const F16Args *fa, co
         u.ay0 = sa.accp.y0;
         u.ay1 = sa.accp.y1;
         u.slot = sa.accp.slot;
-        u.acc = sa.accp.acc;
-        u.cs = sa.src.cs;
-        u.period = sa.src.period;
         u.stage = stage;
     }
     if (fa) {
