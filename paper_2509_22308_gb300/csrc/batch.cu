@@ -435,7 +435,7 @@ __host__ __device__ inline int count_units(int nx, int ny, int seg) {
 // the instances that still run leave warps idle; with every warp busy the long ones are, whose
 // halo rows cost less.
 // (us per step with 16 rows at least / 5: 6 instances of 200^2 7.3 / 5.4, 20 of 136^2 8.1 / 6.2, where two
-// steps per launch take 6.5 and 7.5.)  seg[0] = 0: no four-step launches.
+// steps per launch take 6.5 and 7.5.)  units NULL: no four-step launches.
 constexpr int kUnitLevels = 8;
 struct UnitPlan {
     int seg[kUnitLevels], warps;
@@ -478,14 +478,22 @@ __global__ void __launch_bounds__(1024) k_batch_units(const InstDesc *desc, int 
     build_units(desc, n, t, u);
 }
 
+// The exits of the step before *t_next, without four-step launches.
+__global__ void k_batch_converge(InstDesc *desc, double *energy, double *prev, int *settled,
+                                 const long long *__restrict__ t_next, double tol, int min_periods, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) converge(desc[i], nullptr, energy, prev, settled, *t_next - 1, tol, min_periods, i);
+}
+
 // One block: the exits of the step before *t_next, then the units of the instances that still run, if any has
 // ended since the last listing (listing one instance of 200^2 takes longer than its one-step launch, and
 // with periods of 8 steps every second launch is followed by this kernel).
-__global__ void __launch_bounds__(1024) k_batch_converge(InstDesc *desc, StreamInst *si, double *energy, double *prev,
-                                                         int *settled, const long long *__restrict__ t_next, double tol,
-                                                         int min_periods, int n, const UnitPlan u) {
+__global__ void __launch_bounds__(1024) k_batch_converge_units(InstDesc *desc, StreamInst *si, double *energy,
+                                                               double *prev, int *settled,
+                                                               const long long *__restrict__ t_next, double tol,
+                                                               int min_periods, int n, const UnitPlan u) {
     const long long t = *t_next - 1;
-    const long long listed = u.seg[0] > 0 ? *u.listed : t + 1;
+    const long long listed = *u.listed;
     bool ended = false;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         converge(desc[i], si, energy, prev, settled, t, tol, min_periods, i);
@@ -814,9 +822,13 @@ static cudaError_t batch_launch(lbm_em_batch *b, cudaStream_t s, int p, bool acc
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && b->conv_tol > 0.0 && !b->four) {  // (no period boundary inside a four-step launch)
-        k_batch_converge<<<1, std::min(1024, (b->n + 31) / 32 * 32), 0, s>>>(
-            b->d_desc, b->d_sinsts, b->d_energy, b->d_prev, b->d_settled, b->d_time + (1 - p), b->conv_tol,
-            b->min_periods, b->n, b->units);
+        if (b->units.units)  // the steps at period boundaries between four-step launches
+            k_batch_converge_units<<<1, std::min(1024, (b->n + 31) / 32 * 32), 0, s>>>(
+                b->d_desc, b->d_sinsts, b->d_energy, b->d_prev, b->d_settled, b->d_time + (1 - p), b->conv_tol,
+                b->min_periods, b->n, b->units);
+        else
+            k_batch_converge<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_desc, b->d_energy, b->d_prev, b->d_settled,
+                                                               b->d_time + (1 - p), b->conv_tol, b->min_periods, b->n);
         e = cudaGetLastError();
     }
     return e;
