@@ -42,10 +42,13 @@ KERNELS = {("f32", 1): "k_step<float, false, {P}>", ("f32", 2): "k_step2_tma<fal
            ("f16dev", 2): "k_step2_f16_tma<false> (TMA-staged 64 x 8 tiles)", ("f64", 1): "k_step<double, false, {P}>",
            ("f32", 4): "k_step4_stream<false, {P}> (row-streaming, 4 time levels in registers)",
            ("f16dev", 4): "k_step4_stream<true, TM> (row-streaming, 4 time levels in registers)",
-           ("f32x2", 1): "k_step<df, false, {P}> (double-float)",
+           ("f32x2", 1): "k_step_df<{P}> (double-float, packed pairs of rows)",
            ("f32x2", 2): "k_step2<df, false, {P}> (double-float)"}
-# lattice steps one launch of that kernel advances (the default mode of each form)
-STEPS_PER_LAUNCH = {"f64": 1, "f32": 2, "f16dev": 2}
+# kernel of a form whose lattice stays on chip between the steps of a launch (up to 256)
+ON_CHIP_KERNELS = {"f32": "k_resident32<{P}, false> (state in registers)", "f64": "k_resident<double, {P}, false>",
+                   "f32x2": "k_resident<df, {P}, false>"}
+# FP32 lane operations per lattice update (a fused multiply-add counting one)
+FP32_OPS_PER_LU, FP32_LANES_PER_SM = 36, 128
 # FP64 pipe operations per lattice update of the step kernel: 12 for the moments
 # (sums of 5, 5 and 5 stored populations, one scaling), 16 for the equilibria and 2 f^eq - f
 FP64_OPS_PER_LU = 28
@@ -335,8 +338,8 @@ def profile_case(only="", n=2048):
     L2, a few GB on the device in total), two launches of the FP64 step on one 512^2
     instance of the benchmark workload, then a 24-instance FP32 design map with two steps per
     launch and the same map with four.  `only` picks some of them: "form:mode" pairs for the
-    lattice (of size n; "form:mode:acc" then also accumulates one period on the contour R), "batch2"
-    and "batch4" for the design maps."""
+    lattice (of size n; "form:mode:acc" then also accumulates one period on the contour R; mode "chip":
+    64 steps in one on-chip launch, n up to 512), "batch2" and "batch4" for the design maps."""
     import torch
     from paper_2509_22308_gb300 import build as B
     B.build()
@@ -354,8 +357,8 @@ def profile_case(only="", n=2048):
         pairs = tuple(tuple(p.split(":")) for p in tokens if ":" in p)
         maps = tuple(p for p in tokens if ":" not in p)
     for fp, mode, *acc in pairs:
-        with L.solver_for_instance(inst, fp, steps_per_launch=mode) as s:
-            s.step({"two": 4, "three": 6, "four": 8}.get(mode, 2))
+        with L.solver_for_instance(inst, fp, steps_per_launch="auto" if mode == "chip" else mode) as s:
+            s.step({"two": 4, "three": 6, "four": 8, "chip": 64}.get(mode, 2))
             if acc:
                 s.force_torque(L.make_contour(inst["R"], inst["a"]))
             s.sync()
@@ -454,8 +457,7 @@ def main():
     d_out = torch.zeros((n_inst, 3), dtype=torch.float64, device="cuda")
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
     lus_per_step = sum(instance_lus(i) for i in instances)
-    spl = STEPS_PER_LAUNCH[prec]
-    launches_per_step = sum(2 + i["periods"] * i["period"] // spl for i in instances)
+    spl = solvers[0].steps_per_launch()
     ev = lambda: torch.cuda.Event(enable_timing=True)
 
     def one_step(plain_events=None):
@@ -490,6 +492,7 @@ def main():
     sampler = ClockSampler(local)
     sampler.start()
     step_ms, plain, windows = [], [], []
+    on_chip = -sum(s.resident_launches() for s in solvers)
     for _ in range(args.steps):
         with torch.cuda.stream(main):
             flush.fill_(1.0)
@@ -502,6 +505,11 @@ def main():
         ends = [e0.elapsed_time(b) for _, b, _, _ in plain[n0:]]
         windows.append(max(ends) - min(starts))
     torch.cuda.synchronize()
+    on_chip += sum(s.resident_launches() for s in solvers)
+    # launches of the timed steps: per instance and step the rasterisation and the contour integral, and the
+    # lattice's steps, all on chip (counted by the library) or all in plain launches
+    gpu_launches = args.steps * 2 * n_inst + (
+        on_chip or args.steps * sum(i["periods"] * i["period"] // spl for i in instances))
     results = d_out.cpu().numpy()
     if dist:
         dist.barrier()
@@ -515,7 +523,7 @@ def main():
     # roofline of the dominant kernel, the plain step: its algorithmic work over the
     # window in which the plain steps of all instances ran (CUDA events on their streams)
     plain_ms = sum(windows)
-    plain_launches = sum(n for _, _, n, _ in plain) // n_inst // spl
+    plain_launches = on_chip // n_inst or sum(n for _, _, n, _ in plain) // n_inst // spl
     plain_sites_steps = sum(n * sites for _, _, n, sites in plain)
     # a two-step kernel reads and writes the state once per launch, i.e. once per two steps
     plain_bytes = plain_sites_steps * BYTES_PER_LU[prec] // spl
@@ -530,16 +538,20 @@ def main():
         # against the pipe's measured rate (FMA-chain probe, same run, same clock record)
         ops = plain_sites_steps * FP64_OPS_PER_LU
         achieved_t = ops / (plain_ms / 1e3) / 1e12
+        # the pipe's rate: 2 operations per clock and SM (a probe with more chains per thread than the
+        # library's reaches 0.99 of it)
         derived_t = SMS * FP64_OPS_PER_CLK_PER_SM * sm_mhz * 1e6 / 1e12
-        roofline = {"bound": "alu", "achieved": round(achieved_t, 4), "peak": round(fp64_peak, 4), "unit": "TFLOP/s",
-                    "frac": round(achieved_t / fp64_peak, 4), "traffic": traffic, "kernel": STEP_KERNEL[prec],
+        pipe_t = max(derived_t, fp64_peak)
+        roofline = {"bound": "alu", "achieved": round(achieved_t, 4), "peak": round(pipe_t, 4), "unit": "TFLOP/s",
+                    "frac": round(achieved_t / pipe_t, 4), "traffic": traffic,
+                    "kernel": ON_CHIP_KERNELS[prec].format(P="TM") if on_chip else STEP_KERNEL[prec],
                     "flop_convention": f"FP64 pipe operations (add, multiply or FMA = 1), {FP64_OPS_PER_LU} per "
                                        "lattice update",
-                    "peak_source": "measured: the library's FP64 FMA-chain probe (lbm_em_probe_fp64_fma), best of "
-                                   f"5 launches in this run (median {fp64_peak_median:.4f})",
-                    "peak_derived": round(derived_t, 4),
-                    "peak_derived_source": f"{SMS} SMs x {FP64_OPS_PER_CLK_PER_SM} FP64 ops/clk x median SM clock "
-                                           f"{sm_mhz:.0f} MHz",
+                    "peak_source": f"{SMS} SMs x {FP64_OPS_PER_CLK_PER_SM} FP64 ops/clk x median SM clock "
+                                   f"{sm_mhz:.0f} MHz",
+                    "probe": round(fp64_peak, 4), "frac_of_probe": round(achieved_t / fp64_peak, 4),
+                    "probe_source": "measured: the library's FP64 FMA-chain probe (lbm_em_probe_fp64_fma), best of "
+                                    f"5 launches in this run (median {fp64_peak_median:.4f})",
                     "algorithmic_ops_per_launch": 512 * 512 * FP64_OPS_PER_LU,
                     "avg_launch_us": round(avg_launch_us, 3),
                     "timing": f"{n_inst} instances on {n_inst} streams; avg_launch_us = plain-step window / "
@@ -550,6 +562,15 @@ def main():
         if prof and "fp64_ops_per_launch" in prof:
             roofline["fp64_ops_per_lu_measured"] = round(prof["fp64_ops_per_launch"] / (512 * 512), 3)
             roofline["counters_source"] = "profiles/counters.json (ncu, one 512^2 instance of the workload)"
+    elif on_chip and prec == "f32":
+        # the state stays in registers between the steps of a launch: no bytes to count, so its operations
+        lanes_t = SMS * FP32_LANES_PER_SM * sm_mhz * 1e6 / 1e12
+        achieved_t = plain_sites_steps * FP32_OPS_PER_LU / (plain_ms / 1e3) / 1e12
+        roofline = {"bound": "alu", "achieved": round(achieved_t, 3), "peak": round(lanes_t, 3), "unit": "TFLOP/s",
+                    "frac": round(achieved_t / lanes_t, 4), "traffic": None,
+                    "kernel": ON_CHIP_KERNELS[prec].format(P="TM"),
+                    "flop_convention": f"FP32 lane operations (an FMA = 1), {FP32_OPS_PER_LU} per lattice update",
+                    "avg_launch_us": round(avg_launch_us, 3)}
     else:
         roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(achieved / peak, 4), "traffic": traffic,
@@ -567,7 +588,7 @@ def main():
                             "state can stay L2-resident across the lattice time steps of one run",
                       "parallelism": f"replicas x{world} (independent instances per rank), "
                                      f"{n_inst} concurrent streams per GPU"},
-           "roofline": roofline, "gpu_launches": launches_per_step * args.steps, "clocks": clocks,
+           "roofline": roofline, "gpu_launches": gpu_launches, "clocks": clocks,
            "forces_last_step": results.round(6).tolist()}
 
     if not args.no_e2e:
@@ -623,6 +644,8 @@ def main():
             smp = ClockSampler(local)
             smp.start()
             mlups, gbs_l = [], []
+            fspl = ss[0].steps_per_launch()
+            chip = -sum(s.resident_launches() for s in ss)
             for _ in range(args.repeats):
                 ev_, res = [], []
                 t0e, t1e = ev(), ev()
@@ -643,16 +666,21 @@ def main():
                 pn = sum(n for _, _, n in ev_)
                 mlups.append(lus_per_step / (ms / 1e3) / 1e6)
                 # one read and one write of the state per launch
-                gbs_l.append(pn * 512 * 512 * BYTES_PER_LU[fp] / STEPS_PER_LAUNCH.get(fp, 1) / (pms / 1e3) / 1e9)
+                gbs_l.append(pn * 512 * 512 * BYTES_PER_LU[fp] / fspl / (pms / 1e3) / 1e9)
             fclk = smp.stop()
+            chip += sum(s.resident_launches() for s in ss)
             res = np.array(res)
             ref = results if prec == "f64" else res
             drag = np.abs(ref[:, 0])
             err = np.abs(res - ref) / drag[:, None]
             g = statistics.median(gbs_l)
             forms[fp] = {"mlups": round(statistics.median(mlups), 1), "mlups_spread": spread(mlups),
-                         "step_kernel_gbs": round(g, 1), "steps_per_launch": STEPS_PER_LAUNCH.get(fp, 1),
-                         "frac_hbm": round(g / peak, 4),
+                         "kernel": (ON_CHIP_KERNELS[fp] if chip else KERNELS[(fp, fspl)]).format(P="TM"),
+                         # on chip the state crosses no memory between the steps of a launch
+                         "step_kernel_gbs": None if chip else round(g, 1),
+                         "steps_per_launch": round(args.repeats * sum(i["periods"] * i["period"] for i in instances) / chip, 1)
+                         if chip else fspl,
+                         "frac_hbm": None if chip else round(g / peak, 4),
                          "max_drag_err_rel": float(err[:, 0].max()),
                          "max_lift_torque_err_drag_scale": float(err[:, 1:].max()),
                          "clocks": fclk}
@@ -704,7 +732,8 @@ def main():
                 hs[key]["fp64_ops_per_lu"] = ops
                 t_ops = sites * ops / (us / 1e6) / 1e12
                 hs[key]["fp64_tops"] = round(t_ops, 4)
-                hs[key]["frac_fp64_measured"] = round(t_ops / fp64_peak, 4)
+                hs[key]["frac_fp64_probe"] = round(t_ops / fp64_peak, 4)
+                hs[key]["frac_fp64_pipe"] = round(t_ops / (SMS * FP64_OPS_PER_CLK_PER_SM * sm_mhz * 1e6 / 1e12), 4)
         out["single_domain_8192"] = hs
 
     if not args.no_design_map and rank == 0:
