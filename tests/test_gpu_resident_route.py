@@ -96,19 +96,21 @@ def test_a_captured_stream_and_steps_in_flight_elsewhere_take_plain_launches():
 
 
 # the handle that is in flight, the on-chip one beside it, and whether that takes on-chip launches meanwhile
-@pytest.mark.parametrize("first,second,resident", [
+BESIDE = [
     (("f16dev", 512, "auto"), ("f32", 512), False), (("f32", 512, "two"), ("f32", 350), False), (("f32", 512, "two"), ("f32", 128), False),
     (("f64", 600, "auto"), ("f64", 256), False), (("f32x2", 512, "auto"), ("f32x2", 200), False),
     (("f32", 400, "auto"), ("f32", 512), True),     # both on chip and of the size that always is
     (("f32", 2048, "auto"), ("f64", 128), True), (("f32", 800, "auto"), ("f64", 256), True),  # four steps per launch
     (("f64", 1100, "auto"), ("f32", 400), True),    # fills the GPU by itself
-    (("f16dev", 256, "auto"), ("f64", 128), True)])  # little in the way of FP64
-@pytest.mark.parametrize("streams", ["own", "caller's", "one"])
+    (("f16dev", 256, "auto"), ("f64", 128), True)]  # little in the way of FP64
+
+
+# (on a caller's stream only FP32 from 330^2 sites on is on chip)
+@pytest.mark.parametrize("first,second,resident,streams", [
+    (*b, st) for b in BESIDE for st in ("own", "caller's", "one") if st == "own" or (b[1][0] == "f32" and b[1][1] >= 330)])
 def test_steps_in_flight_of_other_kinds(first, second, resident, streams):
     import torch
     (prec_a, na, spl), (prec_b, nb) = first, second
-    if streams != "own" and not (prec_b == "f32" and nb >= 330):
-        pytest.skip("plain on a caller's stream")
     st = {"own": [None, None], "caller's": [torch.cuda.Stream(), torch.cuda.Stream()], "one": [torch.cuda.Stream()] * 2}[streams]
     j, src = L.make_janus(20.0, 0.4, 2.0, 3.0), L.make_source(24)
     with L.Solver(na, na, prec_a, janus=j, source=src, stream=st[0], steps_per_launch=spl) as a, \
