@@ -78,14 +78,18 @@ typedef enum {
 } lbm_em_source_kind;
 
 /* lbm_em_grid.flags: how many time steps one kernel launch advances.  By default FP64 and
- * double-float advance one step per launch; FP32 two below 2^19 sites and FP16-deviation below
- * 2^20 (each tile and its halo are copied to shared memory by the TMA unit and advance two
- * steps there), four from there on (each warp streams a strip of the lattice through four time
- * levels held in registers).  Runs of FP64, FP32 and double-float lattices small enough to stay
- * on chip (about 550^2, 600^2 and 350^2 sites) take up to 256 steps in one cooperative launch
- * instead: FP32 from 330^2 sites on always, the others on the library's own stream while no
- * other such handle has steps in flight.  The flags force a mode and rule that out.  In FP32, FP64 and double-float the
- * result does not depend on the choice: every mode gives the same bits.  In FP16-deviation the
+ * double-float advance one step per launch; FP32 two below 2^19 sites (narrow lattices, whose
+ * strips would be half empty, below 2^20) and FP16-deviation below 2^20 (each tile and its halo
+ * are copied to shared memory by the TMA unit and advance two steps there), four from there on
+ * (each warp streams a strip of the lattice through four time levels held in registers).
+ * Runs of at least three steps of FP64, FP32 and double-float lattices small enough to stay on
+ * chip (about 550^2, 600^2 and 350^2 sites) take up to 256 steps in one cooperative launch
+ * instead, which needs the whole GPU: FP32 from 330^2 sites on on any stream, the others on the
+ * library's own stream while no other on-chip handle of theirs has steps in flight, and all of
+ * them only while no handle whose plain launches would share the GPU with theirs has steps in
+ * flight on another stream.  The flags force a mode and rule that out.  In FP32, FP64 and
+ * double-float the result does not depend on the choice: every mode gives the same bits.  In
+ * FP16-deviation the
  * four-step mode rounds the stored state to FP16 once per launch instead of once per step, so
  * its bits differ from the other modes by FP16 rounding noise (its runs still give the same
  * bits however they are split, as long as the splits fall on multiples of four steps).
@@ -389,12 +393,15 @@ typedef struct {
                                 4 (FP32, conv_tol 0, nothing else pinned): one warp per work
                                 unit streams a strip of 56 columns and a row segment of an
                                 instance through four time levels held in registers (the
-                                autotuner picks the segment height, 64, 128 or 256 rows); same
-                                bits as one step per launch.  2: the TMA tile kernel above.  With 0 the
-                                autotuner times every kind that applies; with conv_tol > 0
-                                (FP32, nothing pinned) that is the four-step kernel for the
-                                steps between the period boundaries and the one-step kernel
-                                at them, unless many different periods leave few such gaps  */
+                                autotuner picks the segment height of the full batch, 64, 128
+                                or 256 rows; the segments get shorter, down to 5 rows, where
+                                warps would be idle); same bits as one step per launch.  2: the
+                                TMA tile kernel above.  With 0 the autotuner times every kind
+                                that applies; with conv_tol > 0 (FP32, nothing pinned) that is
+                                the four-step kernel for the steps between the period
+                                boundaries and the one-step kernel at them, unless short or
+                                many different periods leave less than 5/8 of the steps in
+                                such gaps                                                  */
 } lbm_em_batch_opts;
 
 typedef struct lbm_em_batch lbm_em_batch_t;

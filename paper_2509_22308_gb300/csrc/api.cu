@@ -645,8 +645,8 @@ static std::vector<MatT<T>> material_table(const double *eps, const bool *pec) {
 // FP16-deviation and FP32 from 2^20 sites on, and of FP32 below that from 2^19 sites on where the strips
 // are well filled (measured on GB300, us per step four / two steps per launch, FP32: 640^2 5.3 / 4.9,
 // 700^2 5.3 / 5.3, 768^2 5.6 / 5.8, 900 x 800 6.4 / 6.7, 1024^2 7.4 / 8.8, 1536^2 12.1 / 20.3; GLUPS at
-// 8192^2 267.9 / 136.8; FP16-deviation, whose bits depend on the steps per launch: GLUPS 8192^2 277.7
-// / 116.8, 1024^2 135 / 99; three steps per launch never led: FP32 8192^2 143.9, 1024^2 111.1 GLUPS:
+// 8192^2 275 / 137; FP16-deviation, whose bits depend on the steps per launch: GLUPS 8192^2 287
+// / 117, 1024^2 135 / 99; three steps per launch never led: FP32 8192^2 144, 1024^2 111 GLUPS:
 // on small lattices the strips cannot fill the GPU and the two-step kernel's state stays in L2).
 // A strip yields 56 columns and a tile of the two-step kernel is 64 x 8, so a narrow lattice can need up to
 // twice as many strips as tiles along x, and then takes four steps per launch only when its tiles cover

@@ -3,8 +3,8 @@
 // separately rounded FP32 operations per instruction).
 //
 // They run at the scalar instructions' lane rate (measured on GB300: 125 against 124 operations
-// per clock and SM) but take half the issue slots, and issue bounds the FP32 kernels that keep
-// the state on chip.  Pairs stay in 64-bit registers throughout: with float2 structs the compiler
+// per clock and SM) but take half the issue slots, and the FP32 kernels that use them are bound by how
+// many instructions a warp has to get through one after the other, not by the pipe.  Pairs stay in 64-bit registers throughout: with float2 structs the compiler
 // moved halves about (one update in a loop: 46 instructions and 135 clocks of latency as float2,
 // 39 and 94 as below; 72 clocks of the FP32 pipe either way; scalar: 73 instructions, 171 clocks).
 // Each half is rounded as the scalar operation, and every expression below is the one of

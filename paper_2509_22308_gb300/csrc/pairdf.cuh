@@ -1,7 +1,8 @@
 // Double-float arithmetic (df32.cuh) on two sites at once with packed FP32 instructions: the operations,
 // their order and so the results are df's (up to the sign of zeros).  A packed instruction works
 // through the pipe at the scalar rate per site but takes one issue slot for two; a double-float
-// update is 540 of them and hardly anything else, so the scalar kernel was bound by issue.
+// update is 536 of them (TM; the scalar form's expressions 652) and hardly anything else, so the scalar
+// kernel was bound by issue.
 #pragma once
 
 #include "common.cuh"

@@ -1081,7 +1081,7 @@ cudaError_t resident_plan(int nx, int ny, int pol, ResidentPlan *plan) {
             fits = p.warps + p.comm <= kResidentMaxWarps && p.rows <= kResidentMaxRows && p.smem <= (size_t)smem_max;
             if (fits) break;
         }
-        // double-float (576 FP32 operations per site) is bound by their latency at the few warps that the
+        // double-float (536 FP32 operations per site) is bound by their latency at the few warps that the
         // registers leave, so with more than one pair of rows per warp the one-step kernel is the faster one
         // (us per step here / there: 256^2 3.7 / 4.7, 320^2 4.0 / 4.8, 384^2 6.3 / 5.6, 512^2 9.0 / 8.0)
         if (std::is_same<T, df>::value && p.rows > 2) fits = false;
