@@ -445,7 +445,8 @@ static lbm_em_status build_graph(lbm_em *h, bool acc, cudaGraphExec_t *out) {
 // 15 / 12, 256^2 18.2 / 16.5, 512^2 18.5 / 17.8; double-float 256^2 42 / 18).  So FP32 lattices of at
 // least kResidentAlways sites take resident launches beside others of the on-chip kind, the rest of
 // that kind only on the library's own stream and while no other of them has steps in flight; a caller's
-// stream keeps its plain launches.  The bits are the same either way.
+// stream keeps its plain launches, because what else the caller runs beside them, on streams that the
+// library does not know, would wait for the whole GPU.  The bits are the same either way.
 //
 // Beside a handle that has plain launches in flight on another stream, an on-chip handle takes plain ones
 // too if that one leaves it room (ms for 1920 steps of each, plain / resident: FP32 512^2 + FP16-deviation
