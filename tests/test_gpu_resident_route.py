@@ -120,7 +120,7 @@ def test_steps_in_flight_of_other_kinds(first, second, resident, streams):
         b.sync()
         n = b.resident_launches()
         assert n == 1
-        a.step(9600)  # tens of milliseconds
+        a.step(20000)  # 25 ms and more
         b.step(48)
         ref.step(96)
         assert b.resident_launches() - n == int(resident or streams == "one")  # (one stream: nothing runs beside it)
